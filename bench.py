@@ -291,9 +291,10 @@ def run_reference(args):
 
 
 # -------------------------------------------------------------- GPU arm --
-# The translation unit of the fused 2D pipeline kernels and the headers it
-# includes: the recorded DRAM traffic stays valid while these are unchanged.
-PIPELINE_SOURCES = ("rve_solver.cu", "rve_colsolve.cuh", "rve_common.cuh", "rve_device.cuh",
+# The translation units of the fused 2D pipeline kernels and the headers they
+# include: the recorded DRAM traffic stays valid while these are unchanged.
+PIPELINE_SOURCES = ("rve_solver.cu", "rve_pipe32.cu", "rve_fused.cuh", "rve_pipeline.cuh",
+                    "rve_colsolve.cuh", "rve_common.cuh", "rve_device.cuh", "rve_fixed.cuh",
                     "rve_internal.h")
 
 

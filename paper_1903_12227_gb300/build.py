@@ -18,7 +18,8 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 LIB = os.path.join(HERE, "librve.so")
 BUILD_DIR = os.path.join(HERE, "_build")
-SOURCES = ["rve_api.cu", "rve_ops.cu", "rve_solver.cu", "rve_plain.cu", "rve_noalloc.cu",
+SOURCES = ["rve_api.cu", "rve_ops.cu", "rve_solver.cu", "rve_pipe32.cu", "rve_pipe64.cu",
+           "rve_persist32.cu", "rve_persist64.cu", "rve_plain.cu", "rve_noalloc.cu",
            "rve_plan.cu", "rve3d.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
@@ -45,9 +46,9 @@ def needs_build() -> bool:
 
 def _compile(src: str, extra: list) -> str:
     obj = os.path.join(BUILD_DIR, os.path.splitext(src)[0] + ".o")
-    # the solver's size dispatch uses templated lambdas (C++20); the other
+    # the pipeline's size dispatch uses templated lambdas (C++20); the other
     # units stay C++17
-    std = "-std=c++20" if src == "rve_solver.cu" else "-std=c++17"
+    std = "-std=c++20" if src.startswith(("rve_solver", "rve_pipe", "rve_persist")) else "-std=c++17"
     cmd = [nvcc(), *ARCH, "-O3", "-lineinfo", std, "-Xcompiler", "-fPIC",
            "-I", INCLUDE, "-I", CSRC, "-c", os.path.join(CSRC, src), "-o", obj, *extra]
     r = subprocess.run(cmd, capture_output=True, text=True)

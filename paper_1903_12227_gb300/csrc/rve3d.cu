@@ -1227,7 +1227,7 @@ struct Plan3 {
     int64_t parts = 0;         // doubles of partials
     int max_log2n = 5;
     size_t o_desc = 0, o_ids = 0, o_tw64 = 0, o_tw32 = 0, o_lap = 0, o_lap32 = 0, o_rho64 = 0,
-           o_rho32 = 0, o_sc = 0, o_part = 0, o_c32 = 0, o_vec = 0, total = 0;
+           o_rho32 = 0, o_fx8 = 0, o_fx4 = 0, o_sc = 0, o_part = 0, o_c32 = 0, o_vec = 0, total = 0;
 };
 
 static rve_status make_plan3(const rve_realization* r, int32_t batch, Plan3& p) {
@@ -1311,6 +1311,8 @@ static rve_status make_plan3(const rve_realization* r, int32_t batch, Plan3& p) 
     p.o_lap32 = take(sizeof(float) * tab);
     p.o_rho64 = take(sizeof(double) * tab);
     p.o_rho32 = take(sizeof(float) * tab);
+    p.o_fx8 = take(sizeof(int4) * tab);
+    p.o_fx4 = take(sizeof(int4) * tab);
     p.o_sc = take(sizeof(MixScal) * p.desc.size());
     p.o_part = take(sizeof(double) * (size_t)p.parts);
     p.o_c32 = take(sizeof(float) * (size_t)p.nodes);
@@ -1338,6 +1340,8 @@ struct Ws3 {   // device pointers into the workspace
         tb.lap32 = reinterpret_cast<const float*>(w + p->o_lap32);
         tb.rho64 = reinterpret_cast<const double*>(w + p->o_rho64);
         tb.rho32 = reinterpret_cast<const float*>(w + p->o_rho32);
+        tb.fx8 = reinterpret_cast<const int4*>(w + p->o_fx8);
+        tb.fx4 = reinterpret_cast<const int4*>(w + p->o_fx4);
         return tb;
     }
     // launch over the units (or the pair-0 units) of group g, `per` (a power

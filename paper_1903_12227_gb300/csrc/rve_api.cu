@@ -212,6 +212,8 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
     p.o_lap32 = take(sizeof(float) * tab);
     p.o_rho64 = take(sizeof(double) * tab);
     p.o_rho32 = take(sizeof(float) * tab);
+    p.o_fx8 = take(sizeof(int4) * tab);
+    p.o_fx4 = take(sizeof(int4) * tab);
     p.o_state = take(sizeof(RState) * batch);
     p.o_partS = take(sizeof(double) * 2 * (size_t)std::max<int64_t>(p.tilesS, maxnb));
     p.o_partU = take(sizeof(double) * 2 * (size_t)p.tilesU);

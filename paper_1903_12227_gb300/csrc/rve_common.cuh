@@ -172,7 +172,10 @@ struct Tables {
     const float* __restrict__ lap32;
     const double* __restrict__ rho64;   // column-filter root for lambda = lap[m], delta = 0
     const float* __restrict__ rho32;    // (1 at m = 0: the singular column)
+    const int4* __restrict__ fx8;       // tw / 8 and tw / 4 in fixed point (rve_fixed.cuh)
+    const int4* __restrict__ fx4;
 };
+__device__ __forceinline__ FxTw fx_twiddles(const Tables& tb, int n) { return FxTw{tb.fx8 + n, tb.fx4 + n, {}}; }
 template <typename T> __device__ __forceinline__ const T* rho_table(const Tables& tb, int n);
 template <> __device__ __forceinline__ const double* rho_table<double>(const Tables& tb, int n) { return tb.rho64 + n; }
 template <> __device__ __forceinline__ const float* rho_table<float>(const Tables& tb, int n) { return tb.rho32 + n; }

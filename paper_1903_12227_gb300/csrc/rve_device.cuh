@@ -18,12 +18,15 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "rve_fixed.cuh"
+
 namespace rve {
 
 // ---------------------------------------------------------------- types --
 template <typename V> struct ScalarOf;
 template <> struct ScalarOf<float2> { typedef float T; };
 template <> struct ScalarOf<double2> { typedef double T; };
+template <> struct ScalarOf<longlong2> { typedef fx_t T; };   // fixed point (rve_fixed.cuh)
 
 template <typename V> __device__ __forceinline__ V mk(typename ScalarOf<V>::T x,
                                                        typename ScalarOf<V>::T y);
@@ -377,17 +380,23 @@ template <typename V> __device__ __forceinline__ void dft4(V& u0, V& u1, V& u2, 
     u3 = csub(d02, d13);
 }
 
+// v / sqrt(2)
+__device__ __forceinline__ float times_rsqrt2(float v) { return 0.70710678118654752440084436210484903928f * v; }
+__device__ __forceinline__ double times_rsqrt2(double v) { return 0.70710678118654752440084436210484903928 * v; }
+__device__ __forceinline__ fx_t times_rsqrt2(fx_t v) { return fx_rsqrt2(v); }
+
 template <typename V> __device__ __forceinline__ void dft8(V* u) {
-    typedef typename ScalarOf<V>::T T;
-    const T c = (T)0.70710678118654752440084436210484903928;
     V e0 = u[0], e1 = u[2], e2 = u[4], e3 = u[6];
     V o0 = u[1], o1 = u[3], o2 = u[5], o3 = u[7];
     dft4(e0, e1, e2, e3);
     dft4(o0, o1, o2, o3);
     // twiddles W8^s = exp(-i pi s/4): 1, c(1-i), -i, -c(1+i)
-    V t1 = mk<V>(c * (o1.x + o1.y), c * (o1.y - o1.x));
+    V t1, t3;
+    t1.x = times_rsqrt2(o1.x + o1.y);
+    t1.y = times_rsqrt2(o1.y - o1.x);
     V t2 = cmul_mi(o2);
-    V t3 = mk<V>(c * (o3.y - o3.x), -c * (o3.x + o3.y));
+    t3.x = times_rsqrt2(o3.y - o3.x);
+    t3.y = -times_rsqrt2(o3.x + o3.y);
     u[0] = cadd(e0, o0); u[4] = csub(e0, o0);
     u[1] = cadd(e1, t1); u[5] = csub(e1, t1);
     u[2] = cadd(e2, t2); u[6] = csub(e2, t2);
@@ -423,7 +432,7 @@ enum { FFT_TO_SMEM = 0, FFT_TO_REGS = 1, FFT_TO_BOTH = 2 };
 //                trailing barrier;
 //   FFT_TO_BOTH: both, then a barrier.
 // Threads with active == false only take part in the barriers.
-// tw[m] = exp(-2 pi i m/n).
+// tw: exp(-2 pi i m/n) by m.
 // LOG2N > 0 makes the size a compile-time constant: the stages unroll and
 // every index folds to an immediate; LOG2N == 0 takes log2n at run time.
 // BS: element x of the sequence sits at buf[pidx(x) * BS], so that BS
@@ -432,12 +441,27 @@ enum { FFT_TO_SMEM = 0, FFT_TO_REGS = 1, FFT_TO_BOTH = 2 };
 // The barriers between stages come from `bar` (default: the whole block;
 // a row team's own barrier when every row is transformed by its own threads,
 // see TeamBar).
+// Fixed-point rows (V = longlong2, TW = FxTw) are divided by powers of two
+// between the stages, with the twiddles or by a shift (rve_fixed.cuh).
+struct FxTw {
+    const int4* __restrict__ w8;   // w / 8
+    const int4* __restrict__ w4;   // w / 4
+    FxShifts f;
+    __device__ __forceinline__ int shift(int stage) const { return stage == 1 ? f.s2 : stage == 2 ? f.s3 : f.s4; }
+};
+__device__ __forceinline__ float2 twiddled(float2 v, const float2* __restrict__ tw, int m, int) { return cmul(v, tw[m]); }
+__device__ __forceinline__ double2 twiddled(double2 v, const double2* __restrict__ tw, int m, int) { return cmul(v, tw[m]); }
+__device__ __forceinline__ longlong2 twiddled(longlong2 v, const FxTw& tw, int m, int stage) {
+    return cmul(v, __ldg((tw.shift(stage) == 3 ? tw.w8 : tw.w4) + m));
+}
+template <typename V, typename TW> __device__ __forceinline__ V untwiddled(V v, const TW&, int) { return v; }
+__device__ __forceinline__ longlong2 untwiddled(longlong2 v, const FxTw& tw, int stage) { return fx_shift(v, tw.shift(stage)); }
 struct BlockBar {
     __device__ __forceinline__ void operator()() const { __syncthreads(); }
 };
-template <int FINAL, int LOG2N = 0, int BS = 1, typename V, typename Bar = BlockBar>
-__device__ __forceinline__ void fft_reg(V (&v)[8], V* buf, int log2n_rt, int t,
-                                        const V* __restrict__ tw, bool active, Bar bar = Bar()) {
+template <int FINAL, int LOG2N = 0, int BS = 1, typename V, typename TW, typename Bar = BlockBar>
+__device__ __forceinline__ void fft_reg(V (&v)[8], V* buf, int log2n_rt, int t, TW tw, bool active,
+                                        Bar bar = Bar()) {
     const int log2n = LOG2N ? LOG2N : log2n_rt;
     const int T = 1 << (log2n - 3);
     const int nstages = (log2n + 2) / 3;   // radix 8, then one radix-4 or -2 tail
@@ -457,8 +481,9 @@ __device__ __forceinline__ void fft_reg(V (&v)[8], V* buf, int log2n_rt, int t,
             if (lr == 3) {
                 const int k = t & (Ns - 1);
                 if (Ns > 1) {
+                    v[0] = untwiddled(v[0], tw, stage);
 #pragma unroll
-                    for (int r = 1; r < 8; ++r) v[r] = cmul(v[r], tw[(r * k) << twshift]);
+                    for (int r = 1; r < 8; ++r) v[r] = twiddled(v[r], tw, (r * k) << twshift, stage);
                 }
                 dft8(v);   // outputs stay in v[r]: the last stage's slots
                 if (to_smem) {
@@ -473,9 +498,10 @@ __device__ __forceinline__ void fft_reg(V (&v)[8], V* buf, int log2n_rt, int t,
                     const int j = t + b * T, k = j & (Ns - 1);
                     V a0 = v[b], a1 = v[b + 2], a2 = v[b + 4], a3 = v[b + 6];
                     if (Ns > 1) {
-                        a1 = cmul(a1, tw[k << twshift]);
-                        a2 = cmul(a2, tw[(2 * k) << twshift]);
-                        a3 = cmul(a3, tw[(3 * k) << twshift]);
+                        a0 = untwiddled(a0, tw, stage);
+                        a1 = twiddled(a1, tw, k << twshift, stage);
+                        a2 = twiddled(a2, tw, (2 * k) << twshift, stage);
+                        a3 = twiddled(a3, tw, (3 * k) << twshift, stage);
                     }
                     dft4(a0, a1, a2, a3);
                     o[b] = a0; o[b + 2] = a1; o[b + 4] = a2; o[b + 6] = a3;
@@ -497,7 +523,10 @@ __device__ __forceinline__ void fft_reg(V (&v)[8], V* buf, int log2n_rt, int t,
                 for (int b = 0; b < 4; ++b) {
                     const int j = t + b * T, k = j & (Ns - 1);
                     V a0 = v[b], a1 = v[b + 4];
-                    if (Ns > 1) a1 = cmul(a1, tw[k << twshift]);
+                    if (Ns > 1) {
+                        a0 = untwiddled(a0, tw, stage);
+                        a1 = twiddled(a1, tw, k << twshift, stage);
+                    }
                     dft2(a0, a1);
                     o[b] = a0; o[b + 4] = a1;
                     if (to_smem) {
@@ -552,6 +581,141 @@ template <typename V> __device__ __forceinline__ V hartley_pair(V zk, V zm) {
     typedef typename ScalarOf<V>::T T;
     const T hf = (T)0.5;
     return mk<V>(hf * ((zk.x + zm.x) - (zk.y - zm.y)), hf * ((zk.y + zm.y) + (zk.x - zm.x)));
+}
+
+// Fixed point: twice (H_a(k), H_b(k)).
+__device__ __forceinline__ longlong2 hartley_pair2(longlong2 zk, longlong2 zm) {
+    longlong2 r;
+    r.x = (zk.x + zm.x) - (zk.y - zm.y);
+    r.y = (zk.y + zm.y) + (zk.x - zm.x);
+    return r;
+}
+
+// Maximum / sum of a value over the T = n/8 threads of a row team.  `scratch`
+// (shared): one word per warp of the block, used by teams of more than one
+// warp; the team's barriers keep successive uses apart.
+template <int T>
+__device__ __forceinline__ unsigned team_max(unsigned v, unsigned* scratch, const TeamBar& bar) {
+    if (T >= 32) {
+        v = __reduce_max_sync(0xffffffffu, v);
+    } else {
+#pragma unroll
+        for (int o = T / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    }
+    if (T > 32) {
+        const int w = threadIdx.x >> 5, w0 = w & ~(T / 32 - 1);
+        if ((threadIdx.x & 31) == 0) scratch[w] = v;
+        bar();
+#pragma unroll
+        for (int k = 0; k < T / 32; ++k) v = max(v, scratch[w0 + k]);
+        bar();   // before the next use
+    }
+    return v;
+}
+template <int T>
+__device__ __forceinline__ unsigned team_sum(unsigned v, unsigned* scratch, const TeamBar& bar) {
+    if (T >= 32) {
+        v = __reduce_add_sync(0xffffffffu, v);
+    } else {
+#pragma unroll
+        for (int o = T / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    }
+    if (T > 32) {
+        const int w = threadIdx.x >> 5, w0 = w & ~(T / 32 - 1);
+        if ((threadIdx.x & 31) == 0) scratch[w] = v;
+        bar();
+        v = 0;
+#pragma unroll
+        for (int k = 0; k < T / 32; ++k) v += scratch[w0 + k];
+        bar();
+    }
+    return v;
+}
+
+// The FP64 form of hartley_row, any size.
+static __device__ __noinline__ void hartley_row_fp64(double2* w, double2* buf, int log2n, int t,
+                                              const double2* __restrict__ tw, bool active,
+                                              TeamBar bar) {
+    const int n = 1 << log2n, T = n >> 3;
+    double2 v[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) v[m] = w[m];
+    fft_reg<FFT_TO_BOTH>(v, buf, log2n, t, tw, active, bar);
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+        if (active) w[m] = hartley_pair(v[m], buf[pidx((n - (t + m * T)) & (n - 1))]);
+}
+
+// Hartley transform of a row of double pairs held by its team (v[m] = element
+// t + m T on entry, the transform's element t + m T on return), through the
+// row's padded buffer: in fixed point where the row allows it (rve_fixed.cuh),
+// else in FP64.  Per pass over 25 x 512^2 nodes (k_row_hartley): 493 us in
+// FP64, at 78 % of the FP64 pipe; 129 us in fixed point, bound by the integer
+// and shared-memory instructions.  Teams that share a warp decide together.  Every thread of
+// the team calls it (active == false: barriers only); on return the mirror
+// reads of `buf` may still be under way in the team's other threads.
+template <int LOG2N>
+__device__ __forceinline__ void hartley_row(double2 (&v)[8], double2* buf, int t,
+                                            const double2* __restrict__ tw, FxTw fx, bool active,
+                                            unsigned* scratch, const TeamBar& bar) {
+    constexpr int n = 1 << LOG2N, T = n / 8;
+    unsigned hi = 0;
+    if (active) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+            hi = max(hi, max((unsigned)__double2hiint(v[m].x) & 0x7FFFFFFFu,
+                             (unsigned)__double2hiint(v[m].y) & 0x7FFFFFFFu));
+    }
+    unsigned E = team_max<T>(hi, scratch, bar) >> 20;
+    bool fixed = !active || fx_takes(E);
+    if (T < 32) fixed = __all_sync(0xffffffffu, fixed);
+    if (fixed) {
+        unsigned size = 0;
+        if (LOG2N >= 7) {
+            if (active) {
+#pragma unroll
+                for (int m = 0; m < 8; ++m)
+                    size += fx_size((unsigned)__double2hiint(v[m].x), E) + fx_size((unsigned)__double2hiint(v[m].y), E);
+            }
+            size = team_sum<T>(size, scratch, bar);
+        }
+        fx.f = fx_schedule(LOG2N, size);
+        E -= fx.f.finer;
+        longlong2 f[8];
+        if (active) {
+#pragma unroll
+            for (int m = 0; m < 8; ++m) f[m] = make_longlong2(fx_from(v[m].x, E), fx_from(v[m].y, E));
+        }
+        longlong2* fb = reinterpret_cast<longlong2*>(buf);
+        fft_reg<FFT_TO_BOTH, LOG2N>(f, fb, LOG2N, t, fx, active, bar);
+        if (active) {
+            const int q = (int)E - FX_BITS + fx_scale(LOG2N, fx.f) - 1;   // the pairs come doubled
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+                const longlong2 h = hartley_pair2(f[m], fb[pidx((n - (t + m * T)) & (n - 1))]);
+                v[m] = make_double2(fx_to(h.x, q), fx_to(h.y, q));
+            }
+        }
+    } else {
+        double2 w[8];   // rare: one copy of the code, its operands through memory
+#pragma unroll
+        for (int m = 0; m < 8; ++m) w[m] = v[m];
+        hartley_row_fp64(w, buf, LOG2N, t, tw, active, bar);
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = w[m];
+    }
+}
+template <int LOG2N>
+__device__ __forceinline__ void hartley_row(float2 (&v)[8], float2* buf, int t,
+                                            const float2* __restrict__ tw, FxTw, bool active,
+                                            unsigned*, const TeamBar& bar) {
+    constexpr int n = 1 << LOG2N, T = n / 8;
+    fft_reg<FFT_TO_BOTH, LOG2N>(v, buf, LOG2N, t, tw, active, bar);
+    if (active) {
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+            v[m] = hartley_pair(v[m], buf[pidx((n - (t + m * T)) & (n - 1))]);
+    }
 }
 
 }  // namespace rve
