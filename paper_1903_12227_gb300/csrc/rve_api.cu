@@ -118,11 +118,12 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
         const int64_t nn = (int64_t)r[b].L * r[b].m0;
         if (nn > 0 && nn <= MAX_N) maxn = std::max(maxn, (int)nn);
     }
-    // column blocks: a segment of up to 32 rows per thread in registers;
-    // 128 threads for the mixed path (3 % faster than 256 and 13 % faster
-    // than 512 on 512^2 grids, measured), 512 for FP64 (its shorter
-    // segments need more threads)
-    p.blockC = (p.vbytes == 8) ? 128 : 512;
+    // column blocks: a segment of up to 32 rows per thread in registers.
+    // Mixed: 128 threads (3 % faster than 256 and 13 % faster than 512 on
+    // 512^2 grids, measured), more where 128 would leave a block under eight
+    // columns, whose rows are its memory accesses.  FP64: 256 threads, two
+    // blocks per SM
+    p.blockC = (p.vbytes == 8) ? (maxn > 1024 ? 512 : maxn > 512 ? 256 : 128) : 256;
     {
         int ts_tuned = 0, bc_tuned = 0;
         if (maxn > 0 && tuned_tiles(maxn, o.precision, o.path == RVE_PATH_PERSISTENT ? 1 : 0,
@@ -183,7 +184,8 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
         // pass's streaming; the preconditioner's row passes use the first
         p.smemU = std::max(p.smemU, (size_t)2 * std::min(t.tU, 2048 / n) * seq * vb);
         // segment end / start values (2 per column segment) and the
-        // singular column's sums (2 per segment)
+        // singular column's sums (2 per segment); FP64: segment values, roots
+        // and totals (tC <= 16 segs: within the same space), and those sums
         p.smemC = std::max(p.smemC, (size_t)(2 * t.tC + 2) * segs * vb);
     }
     if (p.smemS > MAX_SMEM || p.smemU > MAX_SMEM || p.smemC > MAX_SMEM) return RVE_EINVAL;

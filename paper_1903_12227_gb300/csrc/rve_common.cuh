@@ -187,11 +187,13 @@ __host__ __device__ __forceinline__ double filter_root(double mu) {
 }
 
 // Column solve geometry: a thread holds one segment of `col_seg_rows` rows
-// of one column in registers (n/16 rows up to n = 512, then 32; at most 16
-// for FP64 pairs), so a column spans n / col_seg_rows threads.
+// of one column in registers, so a column spans n / col_seg_rows threads.
+// FP32 pairs: 8 rows at n = 32, 16 up to n = 256, then 32 (every thread sums
+// the carries of its column's segments, so small grids want few of them).
+// FP64 pairs: n / 16 rows, at most 16 (registers; the carries are scanned by
+// 16 or more lanes).
 __host__ __device__ constexpr int col_seg_rows(int n, int vbytes) {
-    return (vbytes == 16) ? ((n <= 512 ? n / 16 : 32) < 16 ? (n <= 512 ? n / 16 : 32) : 16)
-                          : (n <= 512 ? n / 16 : 32);
+    return (vbytes == 16) ? (n <= 256 ? n / 16 : 16) : (n <= 32 ? 8 : n <= 256 ? 16 : 32);
 }
 template <typename T> __device__ __forceinline__ const T* lap_table(const Tables& tb, int n);
 template <> __device__ __forceinline__ const double* lap_table<double>(const Tables& tb, int n) { return tb.lap + n; }
