@@ -223,7 +223,7 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
     // 8 double-double sums per tile (FP64), or 8 doubles per strip (mixed)
     p.o_partA = take(sizeof(double) * 16 * (size_t)p.tilesA);
     p.o_ctl = take(sizeof(int32_t) * 64);
-    p.o_uscal = take(sizeof(double) * 2 * (size_t)batch);
+    p.o_uscal = take(sizeof(double) * 4 * (size_t)batch);
     p.o_cnt = take(sizeof(int32_t) * (size_t)batch);
     if (need_vectors) {
         const size_t vec = (size_t)p.nodes * p.vbytes;

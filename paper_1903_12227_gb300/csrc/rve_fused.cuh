@@ -7,11 +7,13 @@
 namespace rve {
 
 // One launch per pipeline kernel (the fused path).
+// The refine and the stencil pass share a launch: a refining realization's
+// blocks compute the true residual where the others run the stencil.  (As a
+// launch of its own the refine pass had nothing to do in 9 of 10 steps and its
+// blocks still took 10 us a step at 4600 blocks, 2 us at one.)
 template <typename V, int SCHEME>
-__global__ void __launch_bounds__(256, sizeof(V) == 8 ? 3 : 2) k_fused_R(const Ctx c) { fused_R_tile<V, SCHEME>(c, blockIdx.x); }
-template <typename V, int SCHEME>
-__global__ void __launch_bounds__(256, sizeof(V) == 8 ? 3 : 2) k_fused_S(const Ctx c) {
-    fused_S_tile<V, SCHEME>(c, blockIdx.x);
+__global__ void __launch_bounds__(256, sizeof(V) == 8 ? 3 : 2) k_fused_RS(const Ctx c, int which) {
+    fused_RS_tile<V, SCHEME>(c, blockIdx.x, which);
 }
 template <typename V>
 __global__ void __launch_bounds__(256, sizeof(V) == 8 ? 4 : 2) k_fused_U(const Ctx c) { fused_U_tile<V>(c, blockIdx.x); }
@@ -22,11 +24,16 @@ __global__ void __launch_bounds__(512) k_fused_C(const Ctx c) {
 
 template <typename V, int SCHEME>
 cudaError_t fused_step(const Plan& p, const Ctx& c, cudaStream_t s, cudaEvent_t* ev) {
-    if (ev) cudaEventRecord(ev[0], s);
-    k_fused_R<V, SCHEME><<<p.tilesS, 256, 0, s>>>(c);
-    if (ev) cudaEventRecord(ev[1], s);
-    k_fused_S<V, SCHEME><<<p.tilesS, 256, p.smemS, s>>>(c);
-    if (ev) cudaEventRecord(ev[2], s);
+    if (ev) {   // profiling: the two halves apart
+        cudaEventRecord(ev[0], s);
+        k_fused_RS<V, SCHEME><<<p.tilesS, 256, p.smemS, s>>>(c, DO_REFINE);
+        cudaEventRecord(ev[1], s);
+        k_fused_RS<V, SCHEME><<<p.tilesS, 256, p.smemS, s>>>(c, DO_STENCIL);
+        cudaEventRecord(ev[2], s);
+        note_launch();
+    } else {
+        k_fused_RS<V, SCHEME><<<p.tilesS, 256, p.smemS, s>>>(c, DO_REFINE | DO_STENCIL);
+    }
     k_fused_U<V><<<p.tilesU, 256, p.smemU, s>>>(c);
     if (ev) cudaEventRecord(ev[3], s);
     k_fused_C<V><<<p.tilesC, p.blockC, p.smemC, s>>>(c);
@@ -34,13 +41,13 @@ cudaError_t fused_step(const Plan& p, const Ctx& c, cudaStream_t s, cudaEvent_t*
     const cudaError_t ce = launch_control(p, c, s);
     if (ce != cudaSuccess) return ce;
     if (ev) cudaEventRecord(ev[5], s);
-    note_launch(5);
+    note_launch(4);
     return cudaGetLastError();
 }
 
 template <typename V, int SCHEME>
 cudaError_t set_smem_attrs(const Plan& p) {
-    cudaError_t e = cudaFuncSetAttribute(k_fused_S<V, SCHEME>,
+    cudaError_t e = cudaFuncSetAttribute(k_fused_RS<V, SCHEME>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smemS);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fused_U<V>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -48,6 +48,20 @@ inline __device__ bool grid_sync(int* ctl, unsigned nblocks, unsigned long long 
     return ok != 0;
 }
 
+// Control step of realization b by one warp.
+inline __device__ void persist_control(const Ctx& c, int b) {
+    if (c.st[b].phase == PH_DONE) return;
+    const int tu0 = c.startU[b], tun = c.startU[b + 1] - tu0;
+    const int tc0 = c.startC[b], tcn = c.startC[b + 1] - tc0;
+    double pU[2], pC[2];
+    for (int k = 0; k < 2; ++k) {
+        pU[k] = warp_sum_array(c.partU + 2 * (int64_t)tu0 + k, tun, 2);
+        pC[k] = warp_sum_array(c.partC + 2 * (int64_t)tc0 + k, tcn, 2);
+    }
+    const bool odd = threadIdx.x & 1;
+    control_apply(c, b, odd ? pU[1] : pU[0], odd ? pC[1] : pC[0]);
+}
+
 struct PersistArgs {
     int tilesS, tilesU, tilesC;
     long long max_steps;
@@ -62,8 +76,7 @@ struct PersistArgs {
 // allocation inside the one persistent kernel.
 template <typename V, int SCHEME>
 __device__ __noinline__ void phase_RS(const Ctx& c, int t) {
-    fused_R_tile<V, SCHEME>(c, t);
-    fused_S_tile<V, SCHEME>(c, t);
+    fused_RS_tile<V, SCHEME>(c, t, DO_REFINE | DO_STENCIL);
 }
 template <typename V>
 __device__ __noinline__ void phase_U(const Ctx& c, int t) { fused_U_tile<V>(c, t); }
@@ -82,7 +95,7 @@ __global__ void __launch_bounds__(256, 2) k_persistent(const Ctx c, const Persis
         if (!grid_sync(c.ndone, nb, a.timeout_ns)) return;
         const int warps = blockDim.x >> 5;
         for (int r = blockIdx.x * warps + (threadIdx.x >> 5); r < c.batch; r += nb * warps)
-            control_one(c, r);
+            persist_control(c, r);
         if (!grid_sync(c.ndone, nb, a.timeout_ns)) return;
         if (*reinterpret_cast<volatile int*>(c.ndone) >= c.batch) return;
     }

@@ -12,8 +12,8 @@
 // the transform is orthogonal up to n, r.z = (1/n^2) sum (H(x)H r)^2 / sigma
 // is read off in the transform domain.
 //
-// Fused pipeline (one CG step = three passes over the vectors + a control
-// kernel; both correctors of a realization travel together as a pair):
+// Fused pipeline (one CG step = three passes over the vectors, R or S first,
+// + a control kernel; both correctors of a realization travel together as a pair):
 //   R  (REFINE steps only) r64 = f - A(u + s (x + alpha p)), the true
 //      residual in double words (FP64 for the FP64 path), partial |r64|^2
 //   S  z = inverse row-Hartley(zhat) on the tile + halo rows, p_new = z +
@@ -62,7 +62,7 @@ struct Ctx {
     double* partS;
     double* partU;
     double* partC;
-    double* uscal;     // [batch][2]: the update kernel's step scalars (see finish_S)
+    double* uscal;     // [batch][4]: the update kernel's step scalars and the sums (see finish_S)
     int* tiles_done;   // [batch]: stencil/refine blocks finished this step
     Tables tb;
     CoefSrc cs;
@@ -174,27 +174,23 @@ inline __device__ void finish_S(const Ctx& c, int b, const RState& s, bool refin
     }
     __syncthreads();
     if (!last) return;
-    if (threadIdx.x < 32) {
+    if (threadIdx.x < 64) {   // one warp per corrector
         __threadfence();
+        const int k = threadIdx.x >> 5;
         const int t0 = c.startS[b], nt = c.startS[b + 1] - t0;
-        const double sx = warp_sum_array(c.partS + 2 * (int64_t)t0, nt, 2);
-        const double sy = warp_sum_array(c.partS + 2 * (int64_t)t0 + 1, nt, 2);
-        if (threadIdx.x == 0) {
-            double a0, a1;
+        const double sum = warp_sum_array(c.partS + 2 * (int64_t)t0 + k, nt, 2);
+        if ((threadIdx.x & 31) == 0) {
+            double a;
             if (!refine) {
-                a0 = s.active[0] ? s.rho[0] / sx : 0.0;
-                a1 = s.active[1] ? s.rho[1] / sy : 0.0;
+                a = s.active[k] ? s.rho[k] / sum : 0.0;
             } else {
-                const double nx = sqrt(sx), ny = sqrt(sy);
-                const bool first = (s.refinements == 0);
-                const bool cx = first ? (nx == 0.0) : (nx <= c.tol * s.fnorm[0]);
-                const bool cy = first ? (ny == 0.0) : (ny <= c.tol * s.fnorm[1]);
-                a0 = cx ? 0.0 : 1.0 / nx;
-                a1 = cy ? 0.0 : 1.0 / ny;
+                const double rn = sqrt(sum);
+                const bool conv = (s.refinements == 0) ? (rn == 0.0) : (rn <= c.tol * s.fnorm[k]);
+                a = conv ? 0.0 : 1.0 / rn;
             }
-            c.uscal[2 * b] = a0;
-            c.uscal[2 * b + 1] = a1;
-            c.tiles_done[b] = 0;   // ready for the next step
+            c.uscal[4 * b + k] = a;
+            c.uscal[4 * b + 2 + k] = sum;
+            if (k == 0) c.tiles_done[b] = 0;   // ready for the next step
         }
     }
 }
@@ -381,8 +377,6 @@ __device__ void refine_tile_dw(const Ctx& c, int tile, int b, const RState& s, c
 // REFINE step: r64 = f - A(u + s (x + alpha p)) for the tile's rows, stored
 // (rounded to the vector type) in q, partial |r64|^2 into partS -- in FP64
 // for the FP64 path, in double words for the mixed path (refine_tile_dw).
-// Launched every step next to k_fused_S; blocks of realizations that are
-// not refining return at once.
 template <int SCHEME>
 __device__ void refine_tile_fp64(const Ctx& c, int tile, int b, const RState& s, const RDesc& d) {
     typedef double2 V;
@@ -421,11 +415,7 @@ __device__ void refine_tile_fp64(const Ctx& c, int tile, int b, const RState& s,
 }
 
 template <typename V, int SCHEME>
-__device__ void fused_R_tile(const Ctx& c, int tile) {
-    const int b = find_real(c.startS, c.batch, tile);
-    const RState& s = c.st[b];
-    if (s.phase != PH_REFINE) return;
-    const RDesc d = c.desc[b];
+__device__ __forceinline__ void refine_tile(const Ctx& c, int tile, int b, const RState& s, const RDesc& d) {
     if constexpr (sizeof(V) == 8) {
         // integer cell values of magnitude <= 2^20: sums of up to four of
         // them, scaled by 2, 4 or 3 h (h a power of two), stay below 2^24
@@ -633,15 +623,22 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
     finish_S(c, b, s, false);
 }
 
+// The refine or the stencil tile, by the realization's phase (`which`: 1
+// refine, 2 stencil, 3 both: the profiler times the two apart).
+enum { DO_REFINE = 1, DO_STENCIL = 2 };
 template <typename V, int SCHEME>
-__device__ void fused_S_tile(const Ctx& c, int tile) {
+__device__ void fused_RS_tile(const Ctx& c, int tile, int which) {
     __shared__ double red[64];   // block_sum2 scratch
     __shared__ unsigned fxs[8];  // row teams' reductions
     __shared__ typename ScalarOf<V>::T bsc[6];
     const int b = find_real(c.startS, c.batch, tile);
     const RState& s = c.st[b];
-    if (s.phase != PH_ITER) return;
+    if (s.phase == PH_DONE || !(which & (s.phase == PH_REFINE ? DO_REFINE : DO_STENCIL))) return;
     const RDesc d = c.desc[b];
+    if (s.phase == PH_REFINE) {
+        refine_tile<V, SCHEME>(c, tile, b, s, d);
+        return;
+    }
     dispatch_size(d.log2n, [&]<int LG>() { fused_S_body<V, SCHEME, LG>(c, tile, b, s, d, red, bsc, fxs); });
 }
 
@@ -683,8 +680,8 @@ __device__ __forceinline__ void fused_U_body(const Ctx& c, int blk, int b, const
     if (phase == PH_ITER) {
         // alpha = rho / p.q, formed by the last stencil block (finish_S)
         if (threadIdx.x == 0) {
-            usc[0] = (T)c.uscal[2 * b];
-            usc[1] = (T)c.uscal[2 * b + 1];
+            usc[0] = (T)c.uscal[4 * b];
+            usc[1] = (T)c.uscal[4 * b + 1];
         }
         // rt of the block's rows is read group by group: one thread per row
         // asks for it in L2 now
@@ -751,8 +748,8 @@ __device__ __forceinline__ void fused_U_body(const Ctx& c, int blk, int b, const
                 usc[1] = (float)s.s[1];
                 usc[2] = (float)s.alpha[0];
                 usc[3] = (float)s.alpha[1];
-                usc[4] = (float)c.uscal[2 * b];       // 1 / |r| per corrector (0 once
-                usc[5] = (float)c.uscal[2 * b + 1];   // converged), from finish_S
+                usc[4] = (float)c.uscal[4 * b];       // 1 / |r| per corrector (0 once
+                usc[5] = (float)c.uscal[4 * b + 1];   // converged), from finish_S
             }
             __syncthreads();
         }
@@ -792,7 +789,7 @@ __device__ __forceinline__ void fused_U_body(const Ctx& c, int blk, int b, const
                 }
             } else {   // REFINE, FP64
                 // 1 / |r64| per corrector (0 once converged), from finish_S
-                const double ix = c.uscal[2 * b], iy = c.uscal[2 * b + 1];
+                const double ix = c.uscal[4 * b], iy = c.uscal[4 * b + 1];
                 if (active) {
 #pragma unroll
                     for (int m = 0; m < 8; ++m) {
@@ -882,109 +879,119 @@ __device__ __forceinline__ bool bad(double v) { return !isfinite(v); }
 constexpr double STALL_FACTOR = 0.7;
 constexpr int STALL_STEPS = 30;
 
-// Control step of realization b, executed by one whole warp.
-inline __device__ void control_one(const Ctx& c, int b) {
+// Control step of realization b by one whole warp: lane k < 2 handles
+// corrector k, with pU, pC its sums of the update and column passes.  (FP64
+// square roots and divisions take about a microsecond each here: side by side
+// for the two correctors, and alpha is the one finish_S formed.)
+inline __device__ void control_apply(const Ctx& c, int b, double pU, double pC) {
     RState& s = c.st[b];
-    if (s.phase == PH_DONE) return;
-    const int ts0 = c.startS[b], tsn = c.startS[b + 1] - ts0;
-    const int tu0 = c.startU[b], tun = c.startU[b + 1] - tu0;
-    const int tc0 = c.startC[b], tcn = c.startC[b + 1] - tc0;
-    double pS[2], pU[2], pC[2];
-    for (int k = 0; k < 2; ++k) {
-        pS[k] = warp_sum_array(c.partS + 2 * (int64_t)ts0 + k, tsn, 2);
-        pU[k] = warp_sum_array(c.partU + 2 * (int64_t)tu0 + k, tun, 2);
-        pC[k] = warp_sum_array(c.partC + 2 * (int64_t)tc0 + k, tcn, 2);
-    }
-    if ((threadIdx.x & 31) != 0) return;
+    const int k = threadIdx.x & 31;
+    const bool mine = k < 2;
+    const unsigned upto = k < 2 ? (2u << k) - 1u : 0u;   // correctors 0 .. k
     if (s.phase == PH_ITER) {
-        s.steps += 1;
-        bool any_active = false;
-        for (int k = 0; k < 2; ++k) {
-            if (!s.active[k]) { s.alpha[k] = 0.0; s.beta[k] = 0.0; continue; }
-            const double alpha = s.rho[k] / pS[k];
-            const double rn = sqrt(pU[k]);
-            if (bad(alpha) || bad(rn) || bad(pC[k])) {
-                s.status = RVE_ENAN;
-                s.phase = PH_DONE;
-                atomicAdd(c.ndone, 1);
-                return;
-            }
+        const bool act = mine && s.active[k];
+        const double alpha = act ? c.uscal[4 * b + k] : 0.0;
+        const double rn = act ? sqrt(pU) : 0.0;
+        const unsigned nan = __ballot_sync(0xffffffffu, act && (bad(alpha) || bad(rn) || bad(pC)));
+        bool go = false, last = false;
+        if (mine && !act) {
+            if (!(nan & upto)) { s.alpha[k] = 0.0; s.beta[k] = 0.0; }
+        } else if (act && !(nan & upto)) {
             s.alpha[k] = alpha;
-            s.iters[k] += 1;
+            const int it = s.iters[k] + 1;
+            s.iters[k] = it;
             // a cycle whose residual has stopped falling (the attainable
             // accuracy of the inner precision) ends early: the refinement
             // step then restarts from the true residual
+            bool stalled = false;
             if (rn < STALL_FACTOR * s.best[k]) {
                 s.best[k] = rn;
                 s.stall[k] = 0;
             } else {
-                s.stall[k] += 1;
+                const int st = s.stall[k] + 1;
+                s.stall[k] = st;
+                stalled = st >= STALL_STEPS;
             }
-            const bool stalled = s.stall[k] >= STALL_STEPS;
-            if (rn <= s.target[k] || stalled || s.iters[k] >= c.max_iter) {
+            if (rn <= s.target[k] || stalled || it >= c.max_iter) {
                 s.active[k] = 0;       // frozen; alpha still pending for x
                 s.beta[k] = 0.0;
-                if (s.iters[k] >= c.max_iter && rn > s.target[k]) s.final_pass = 1;
+                last = it >= c.max_iter && rn > s.target[k];
             } else {
-                s.beta[k] = pC[k] / s.rho[k];
-                s.rho[k] = pC[k];
-                any_active = true;
+                s.beta[k] = pC / s.rho[k];
+                s.rho[k] = pC;
+                go = true;
             }
         }
-        s.parity ^= 1;
-        if (!any_active) s.phase = PH_REFINE;   // every corrector ended its cycle
-        return;
-    }
-    // REFINE: true residual of the accumulated solution
-    s.refinements += 1;
-    bool all_done = true;
-    for (int k = 0; k < 2; ++k) {
-        const double rn = sqrt(pS[k]);
-        if (bad(rn)) {
+        const unsigned any = __ballot_sync(0xffffffffu, go), fin = __ballot_sync(0xffffffffu, last);
+        if (k != 0) return;
+        s.steps += 1;
+        if (fin) s.final_pass = 1;
+        if (nan) {
             s.status = RVE_ENAN;
             s.phase = PH_DONE;
             atomicAdd(c.ndone, 1);
             return;
         }
-        if (s.refinements == 1) s.fnorm[k] = rn;
-        const bool conv = (s.refinements == 1) ? (rn == 0.0) : (rn <= c.tol * s.fnorm[k]);
+        s.parity ^= 1;
+        if (!any) s.phase = PH_REFINE;   // every corrector ended its cycle
+        return;
+    }
+    // REFINE: true residual of the accumulated solution
+    const int refs = s.refinements + 1;
+    const double rn = mine ? sqrt(c.uscal[4 * b + 2 + k]) : 0.0;
+    const unsigned nan = __ballot_sync(0xffffffffu, mine && bad(rn));
+    bool open = false, last = false;
+    if (mine && !(nan & upto)) {
+        if (refs == 1) s.fnorm[k] = rn;
+        const double fn = s.fnorm[k];
+        const bool conv = (refs == 1) ? (rn == 0.0) : (rn <= c.tol * fn);
         const double prev = s.relres[k];
-        s.relres[k] = s.fnorm[k] > 0.0 ? rn / s.fnorm[k] : 0.0;
+        const double rel = fn > 0.0 ? rn / fn : 0.0;
+        s.relres[k] = rel;
         s.alpha[k] = 0.0;
-        if (conv || s.cdone[k]) {
-            s.cdone[k] = 1;
-            s.active[k] = 0;
-            s.s[k] = 0.0;
-            s.beta[k] = 0.0;
-            continue;
-        }
-        all_done = false;
         // each cycle restarts CG from the true residual (p = z): keeping
         // the old direction across the replaced residual loses conjugacy
         // when the FP32 recurrence has drifted (tens of percent here)
         s.beta[k] = 0.0;
-        s.s[k] = rn;
-        s.active[k] = 1;
-        s.best[k] = 1.0;   // the inner system starts from r / |r|
-        s.stall[k] = 0;
-        // inner target: what the outer tolerance still needs, but no less
-        // than the usual inner reduction
-        const double want = 0.5 * c.tol * s.fnorm[k] / rn;
-        double tgt = fmax(want, c.inner_tol);
-        // a cycle gains at most what the rounding of its iterate allows
-        // (about eps_inner times the condition of A on the correction): when
-        // the last cycle's true residual fell far less than it was asked
-        // to, ask the next one for no more than ten times what it achieved
-        if (s.refinements >= 2 && prev > 0.0) {
-            const double got = s.relres[k] / prev;
-            if (got > 10.0 * s.target[k]) tgt = fmax(tgt, 0.1 * got);
+        if (conv || s.cdone[k]) {
+            s.cdone[k] = 1;
+            s.active[k] = 0;
+            s.s[k] = 0.0;
+        } else {
+            open = true;
+            s.s[k] = rn;
+            s.active[k] = 1;
+            s.best[k] = 1.0;   // the inner system starts from r / |r|
+            s.stall[k] = 0;
+            // inner target: what the outer tolerance still needs, but no less
+            // than the usual inner reduction
+            const double want = 0.5 * c.tol * fn / rn;
+            double tgt = fmax(want, c.inner_tol);
+            // a cycle gains at most what the rounding of its iterate allows
+            // (about eps_inner times the condition of A on the correction): when
+            // the last cycle's true residual fell far less than it was asked
+            // to, ask the next one for no more than ten times what it achieved
+            if (refs >= 2 && prev > 0.0) {
+                const double got = rel / prev;
+                if (got > 10.0 * s.target[k]) tgt = fmax(tgt, 0.1 * got);
+            }
+            s.target[k] = fmin(0.5, tgt);
+            s.rho[k] = pC;
+            last = s.iters[k] >= c.max_iter;
         }
-        s.target[k] = fmin(0.5, tgt);
-        s.rho[k] = pC[k];
-        if (s.iters[k] >= c.max_iter) s.final_pass = 1;
     }
-    if (all_done || s.final_pass) {
-        if (!all_done) s.status = RVE_ENOCONV;
+    const unsigned any = __ballot_sync(0xffffffffu, open), fin = __ballot_sync(0xffffffffu, last);
+    if (k != 0) return;
+    s.refinements = refs;
+    if (fin) s.final_pass = 1;
+    if (nan) {
+        s.status = RVE_ENAN;
+        s.phase = PH_DONE;
+        atomicAdd(c.ndone, 1);
+        return;
+    }
+    if (!any || s.final_pass) {
+        if (any) s.status = RVE_ENOCONV;
         s.phase = PH_DONE;
         atomicAdd(c.ndone, 1);
         return;
