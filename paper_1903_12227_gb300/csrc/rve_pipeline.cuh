@@ -291,10 +291,14 @@ __device__ void refine_tile_dw(const Ctx& c, int tile, int b, const RState& s, c
         }
     };
     dword nx{0.f, 0.f}, ny{0.f, 0.f};   // |r|^2, double-word per thread
+    // n < 256: 256 / n groups of threads share the tile's rows
+    const int W = min(n, (int)blockDim.x), per = (rows + (int)blockDim.x / W - 1) / ((int)blockDim.x / W);
+    const int q0 = ((int)threadIdx.x / W) * per, q1 = min(rows, q0 + per);
+    const int col = q0 < q1 ? (int)threadIdx.x & (W - 1) : n;
     if (first) {   // u = x = p = 0: r = f, the same arithmetic without the zero terms
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            CW cmm = cell(r0 - 1, j - 1), cm0 = cell(r0 - 1, j);
-            for (int q = 0; q < rows; ++q) {
+        for (int j = col; j < n; j += blockDim.x) {
+            CW cmm = cell(r0 + q0 - 1, j - 1), cm0 = cell(r0 + q0 - 1, j);
+            for (int q = q0; q < q1; ++q) {
                 const int i = r0 + q;
                 const CW c0m = cell(i, j - 1), c00 = cell(i, j);
                 dword kfx, kfy;   // K f
@@ -317,11 +321,12 @@ __device__ void refine_tile_dw(const Ctx& c, int tile, int b, const RState& s, c
             }
         }
     }
-    for (int j = first ? n : threadIdx.x; j < n; j += blockDim.x) {
-        float4 a0 = wat(r0 - 1, j - 1), a1 = wat(r0 - 1, j), a2 = wat(r0 - 1, j + 1);
-        float4 b0 = wat(r0, j - 1), b1 = wat(r0, j), b2 = wat(r0, j + 1);
-        CW cmm = cell(r0 - 1, j - 1), cm0 = cell(r0 - 1, j);
-        for (int q = 0; q < rows; ++q) {
+    for (int j = first ? n : col; j < n; j += blockDim.x) {
+        const int ra = r0 + q0 - 1;
+        float4 a0 = wat(ra, j - 1), a1 = wat(ra, j), a2 = wat(ra, j + 1);
+        float4 b0 = wat(ra + 1, j - 1), b1 = wat(ra + 1, j), b2 = wat(ra + 1, j + 1);
+        CW cmm = cell(ra, j - 1), cm0 = cell(ra, j);
+        for (int q = q0; q < q1; ++q) {
             const int i = r0 + q;
             const float4 e0 = wat(i + 1, j - 1), e1 = wat(i + 1, j), e2 = wat(i + 1, j + 1);
             const CW c0m = cell(i, j - 1), c00 = cell(i, j);
@@ -468,6 +473,10 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
     }
     const int SEQ = seq_stride(n);
     V* Pt = reinterpret_cast<V*>(smem_raw);            // (TR+2) padded rows
+    // a tile of the whole realization: its halo rows are its own last and
+    // first row, stored twice instead of transformed twice
+    const bool whole = LOG2N <= 6 && TR == n;
+    const int s0 = whole ? 1 : 0, slots = whole ? TR : TR + 2;   // slots to transform
     uint32_t* mrows = reinterpret_cast<uint32_t*>(Pt + (TR + 2) * SEQ);
     const int wpr = n >> 5;
     if (!c.cs.coef) {
@@ -489,8 +498,8 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
     // ahead: the copies of group g+1 are in flight while group g transforms
     // and while the stencil runs on the rows group g completed
     auto prefetch = [&](int g0) {
-        const int q = g0 + L.qq;
-        if (g0 < TR + 2 && q < TR + 2) {
+        const int q = s0 + g0 + L.qq;
+        if (g0 + L.qq < slots) {
             const int row = (r0 - 1 + q) & (n - 1);
             V* buf = Pt + q * SEQ;
 #pragma unroll
@@ -513,14 +522,16 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
         T cmm, cm0;
         int j, pm, p0, pp;
     };
-    auto win_start = [&](Win& w, int j) {
+    auto win_start = [&](Win& w, int j, int q0) {   // in front of own slot q0
         w.j = j;
         const int jm = (j - 1) & (n - 1), jp = (j + 1) & (n - 1);
         w.pm = pidx(jm); w.p0 = pidx(j); w.pp = pidx(jp);
-        w.u0 = Pt[w.pm]; w.u1 = Pt[w.p0]; w.u2 = Pt[w.pp];                    // slot 0
-        w.m0 = Pt[SEQ + w.pm]; w.m1 = Pt[SEQ + w.p0]; w.m2 = Pt[SEQ + w.pp];  // slot 1
-        w.cmm = tc.cell(c.cs, d, 0, r0 - 1, jm);
-        w.cm0 = tc.cell(c.cs, d, 0, r0 - 1, j);
+        const V* up = Pt + (q0 - 1) * SEQ;
+        const V* md = up + SEQ;
+        w.u0 = up[w.pm]; w.u1 = up[w.p0]; w.u2 = up[w.pp];
+        w.m0 = md[w.pm]; w.m1 = md[w.p0]; w.m2 = md[w.pp];
+        w.cmm = tc.cell(c.cs, d, q0 - 1, r0 + q0 - 2, jm);
+        w.cm0 = tc.cell(c.cs, d, q0 - 1, r0 + q0 - 2, j);
     };
     auto win_step = [&](Win& w, int q) {   // own slot q: node row r0 + q - 1
         const V* dn = Pt + (q + 1) * SEQ;
@@ -541,13 +552,23 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
         w.m0 = d0; w.m1 = d1; w.m2 = d2;
         w.cmm = c0m; w.cm0 = c00;
     };
+    // n < 256: 256 / n groups of threads share the tile's rows (at n = 64 the
+    // columns alone kept 64 of 256 threads busy)
     auto stencil_rows = [&]() {
         constexpr bool TWO = LOG2N >= 9;   // n >= 512 = 2 x 256 threads
-        for (int j = threadIdx.x; j < n; j += TWO ? 512 : 256) {
+        constexpr int W = LOG2N < 8 ? 1 << LOG2N : 256;
+        int q0 = 1, q1 = TR;
+        if (W < 256) {
+            const int per = (TR + 256 / W - 1) / (256 / W);
+            q0 = 1 + (threadIdx.x / W) * per;
+            q1 = min(TR, q0 + per - 1);
+            if (q0 > q1) return;
+        }
+        for (int j = threadIdx.x & (W - 1); j < n; j += TWO ? 512 : 256) {
             Win wa, wb;
-            win_start(wa, j);
-            if (TWO) win_start(wb, j + 256);
-            for (int q = 1; q <= TR; ++q) {
+            win_start(wa, j, q0);
+            if (TWO) win_start(wb, j + 256, q0);
+            for (int q = q0; q <= q1; ++q) {
                 win_step(wa, q);
                 if (TWO) win_step(wb, q);
             }
@@ -557,9 +578,9 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
     // barriers of the group loop are the team's, so the teams of a block
     // drift independently (one waits on its loads while another transforms)
     const TeamBar team(L.qq, L.z.T);
-    for (int g0 = 0; g0 < TR + 2; g0 += L.G) {
-        const int q = g0 + L.qq;
-        const bool active = q < TR + 2;
+    for (int g0 = 0; g0 < slots; g0 += L.G) {
+        const int q = s0 + g0 + L.qq;
+        const bool active = g0 + L.qq < slots;
         const int row = (r0 - 1 + q) & (n - 1);
         const bool own = active && q >= 1 && q <= TR;
         prefetch(g0 + L.G);
@@ -609,6 +630,11 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
         if (active) {
 #pragma unroll
             for (int m = 0; m < 8; ++m) buf[pidx(L.t + m * L.z.T)] = pn[m];
+            if (whole && (q == 1 || q == TR)) {
+                V* twin = Pt + (q == 1 ? TR + 1 : 0) * SEQ;
+#pragma unroll
+                for (int m = 0; m < 8; ++m) twin[pidx(L.t + m * L.z.T)] = pn[m];
+            }
         }
     }
     cp_async_wait<0>();

@@ -1,0 +1,35 @@
+"""Tile heights follow from the batch's size: solves of one realization, of a
+few and of many, over the grid sizes where whole tiles, row groups and parts of
+a transform group meet, against each other and the true residual."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1903_12227_gb300 import rve, workloads
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("precision", [rve.FP64, rve.MIXED])
+@pytest.mark.parametrize("scheme", [rve.CONSISTENT, rve.LUMPED])
+@pytest.mark.parametrize("n,count", [(32, 300), (64, 300), (128, 40), (256, 9), (512, 3), (1024, 2)])
+def test_lone_and_batched_solves(n, count, scheme, precision):
+    ds = workloads.batch(n // 8, 8, 10.0, 4, count)
+    tol = 1e-10
+    opts = rve.make_opts(scheme=scheme, precision=precision, tol=tol)
+    mask = rve.gen_field(ds)
+    u, info = rve.solve(ds, mask=mask, opts=opts)
+    assert all(i["status"] == rve.RVE_OK for i in rve.info_to_dicts(info, count))
+    f = rve.rhs(ds, mask=mask)
+    r = (f - rve.apply_stiffness(ds, u, mask=mask, scheme=scheme)).view(count, n * n, 2)
+    # the solver's own residual met tol; this one differs by FP64 rounding of
+    # A u (8 eps |A| |u| per node, |A| <= 16 a_max) and, mixed, of the final u
+    floor = 64 * 2.0 ** -53 * 160.0 * u.view(count, -1, 2).abs().amax(1) * n
+    assert bool((r.norm(dim=1) <= tol * f.view(count, n * n, 2).norm(dim=1) + floor).all())
+    A = rve.a_hom(ds, u, mask=mask, scheme=scheme)
+    words = n * n // 32
+    for k in (0, count - 1):   # two answers to the same tolerance: the energies differ by its square
+        m = mask[k * words:(k + 1) * words]
+        v, _ = rve.solve(ds[k:k + 1], mask=m, opts=opts)
+        B = rve.a_hom(ds[k:k + 1], v, mask=m, scheme=scheme)
+        np.testing.assert_allclose(B[0].cpu().numpy(), A[k].cpu().numpy(), rtol=0, atol=1e-10)
