@@ -136,6 +136,102 @@ __device__ __forceinline__ V stencil_apply(const CellsT<typename ScalarOf<V>::T>
     return q;
 }
 
+// A stencil row of FP64 pairs, scaled by K = 6 (consistent) or 2 (lumped) so
+// that its weights are small multiples of cell sums: K A has centre 4 (2) times
+// the sum of the four cells, edges -(sum of the two shared cells), corners -2
+// (0) times the shared cell.  The weights of integer cell values are exact and
+// their row sums vanish.  GB300 issues 2 FP64 operations per clock and SM; with
+// the weights formed from the cells in every row a node took 35 of them.  With
+// the 16 possible rows of a two-valued field in a shared-memory table it takes
+// 18, with explicit cell values 25 (a thread walking down a column forms 5
+// sums per row).
+template <int SCHEME> __host__ __device__ constexpr double row_scale() { return SCHEME == 0 ? 6.0 : 2.0; }
+template <int SCHEME> __device__ __forceinline__ constexpr double row_centre() { return SCHEME == 0 ? 4.0 : 2.0; }
+struct StencilRow { double c, n, w, e, s, mm, m0, om, oo; };   // edges and corners without their signs
+
+constexpr int ROW_STRIDE = 10;   // doubles per table entry (16-byte loads, two-way conflicts at most)
+constexpr int ROW_TABLE = 16 * ROW_STRIDE;
+// Entry b0 + 2 b1 + 4 b2 + 8 b3: cells (i-1,j-1), (i-1,j), (i,j-1), (i,j)
+// covered; corners doubled.  Threads 0 .. 15; no barrier.
+template <int SCHEME>
+__device__ __forceinline__ void fill_row_table(double* tab, double am, double ai) {
+    const int k = threadIdx.x;
+    if (k >= 16) return;
+    const double mm = (k & 1) ? ai : am, m0 = (k & 2) ? ai : am, om = (k & 4) ? ai : am, oo = (k & 8) ? ai : am;
+    double* t = tab + k * ROW_STRIDE;
+    t[0] = row_centre<SCHEME>() * ((mm + m0) + (om + oo));
+    t[1] = mm + m0;
+    t[2] = mm + om;
+    t[3] = m0 + oo;
+    t[4] = om + oo;
+    t[5] = 2.0 * mm;
+    t[6] = 2.0 * m0;
+    t[7] = 2.0 * om;
+    t[8] = 2.0 * oo;
+    t[9] = 0.0;
+}
+template <int SCHEME>
+__device__ __forceinline__ StencilRow table_row(const double* tab, unsigned k) {
+    const double2* t = reinterpret_cast<const double2*>(tab + k * ROW_STRIDE);
+    const double2 a = t[0], b = t[1], c = t[2];
+    StencilRow r{a.x, a.y, b.x, b.y, c.x, c.y, 0.0, 0.0, 0.0};
+    if (SCHEME == 0) {
+        const double2 f = t[3], h = t[4];
+        r.m0 = f.x;
+        r.om = f.y;
+        r.oo = h.x;
+    }
+    return r;
+}
+// Explicit cell values down a column: step(a(i,j-1), a(i,j)) moves to the next
+// row; corners single.
+template <int SCHEME> struct RowWalk {
+    double amm, am0, n;
+    __device__ __forceinline__ RowWalk(double mm, double m0) : amm(mm), am0(m0), n(mm + m0) {}
+    __device__ __forceinline__ StencilRow step(double om, double oo) {
+        StencilRow r;
+        r.n = n;
+        r.s = om + oo;
+        r.w = amm + om;
+        r.e = am0 + oo;
+        r.c = row_centre<SCHEME>() * (r.n + r.s);
+        r.mm = amm;
+        r.m0 = am0;
+        r.om = om;
+        r.oo = oo;
+        amm = om; am0 = oo; n = r.s;
+        return r;
+    }
+};
+// K (A p) at a node (DOUBLED: the row's corners are doubled).
+template <int SCHEME, bool DOUBLED>
+__device__ __forceinline__ double2 apply_row(const StencilRow& r, double2 pmm, double2 pm0, double2 pmp,
+                                             double2 p0m, double2 p00, double2 p0p, double2 ppm,
+                                             double2 pp0, double2 ppp) {
+    double2 q = make_double2(r.c * p00.x, r.c * p00.y);
+    auto sub = [](double2& t, double w, double2 v) {
+        t.x = fma(-w, v.x, t.x);
+        t.y = fma(-w, v.y, t.y);
+    };
+    sub(q, r.n, pm0);
+    sub(q, r.w, p0m);
+    sub(q, r.e, p0p);
+    sub(q, r.s, pp0);
+    if (SCHEME == 0 && DOUBLED) {
+        sub(q, r.mm, pmm);
+        sub(q, r.m0, pmp);
+        sub(q, r.om, ppm);
+        sub(q, r.oo, ppp);
+    } else if (SCHEME == 0) {
+        double2 t = make_double2(r.mm * pmm.x, r.mm * pmm.y);
+        sub(t, -r.m0, pmp);
+        sub(t, -r.om, ppm);
+        sub(t, -r.oo, ppp);
+        sub(q, 2.0, t);
+    }
+    return q;
+}
+
 // Galerkin right-hand sides at a node from its four cells.
 __device__ __forceinline__ double2 rhs_at(const Cells4& a, double h) {
     const double hh = 0.5 * h;

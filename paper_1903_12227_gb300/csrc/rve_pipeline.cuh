@@ -164,7 +164,7 @@ struct TileCoef {
 // stores the update kernel's scalars: in ITER alpha = rho / p.q (0 for a
 // frozen corrector), in REFINE 1/|r64| (0 once the corrector meets the
 // tolerance).  The update kernel then starts without any FP64 work.
-inline __device__ void finish_S(const Ctx& c, int b, const RState& s, bool refine) {
+inline __device__ void finish_S(const Ctx& c, int b, const RState& s, bool refine, double scale) {
     __shared__ int last;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -183,13 +183,14 @@ inline __device__ void finish_S(const Ctx& c, int b, const RState& s, bool refin
             double a;
             if (!refine) {
                 a = s.active[k] ? s.rho[k] / sum : 0.0;
+                c.uscal[4 * b + 2 + k] = scale * a;
             } else {
                 const double rn = sqrt(sum);
                 const bool conv = (s.refinements == 0) ? (rn == 0.0) : (rn <= c.tol * s.fnorm[k]);
                 a = conv ? 0.0 : 1.0 / rn;
+                c.uscal[4 * b + 2 + k] = sum;
             }
             c.uscal[4 * b + k] = a;
-            c.uscal[4 * b + 2 + k] = sum;
             if (k == 0) c.tiles_done[b] = 0;   // ready for the next step
         }
     }
@@ -376,7 +377,7 @@ __device__ void refine_tile_dw(const Ctx& c, int tile, int b, const RState& s, c
         c.partS[2 * (int64_t)tile] = sx;
         c.partS[2 * (int64_t)tile + 1] = sy;
     }
-    finish_S(c, b, s, true);
+    finish_S(c, b, s, true, 1.0);
 }
 
 // REFINE step: r64 = f - A(u + s (x + alpha p)) for the tile's rows, stored
@@ -398,14 +399,15 @@ __device__ void refine_tile_fp64(const Ctx& c, int tile, int b, const RState& s,
         const Cells4 a = cells_at(c.cs, d, i, j);
         const double2 f = load_at(c.cs, d, ((int64_t)i << d.log2n) + j, a);
         double2 Aw = make_double2(0.0, 0.0);
+        constexpr double IK = 1.0 / row_scale<SCHEME>();
         if (!first)
-            Aw = stencil_apply<SCHEME, double2>(
-                a, refine_w(c, d, s, i - 1, j - 1, Pold), refine_w(c, d, s, i - 1, j, Pold),
+            Aw = apply_row<SCHEME, false>(
+                RowWalk<SCHEME>(a.mm, a.m0).step(a.z0m, a.z00), refine_w(c, d, s, i - 1, j - 1, Pold), refine_w(c, d, s, i - 1, j, Pold),
                 refine_w(c, d, s, i - 1, j + 1, Pold), refine_w(c, d, s, i, j - 1, Pold),
                 refine_w(c, d, s, i, j, Pold), refine_w(c, d, s, i, j + 1, Pold),
                 refine_w(c, d, s, i + 1, j - 1, Pold), refine_w(c, d, s, i + 1, j, Pold),
                 refine_w(c, d, s, i + 1, j + 1, Pold));
-        const double2 r64 = make_double2(f.x - Aw.x, f.y - Aw.y);
+        const double2 r64 = make_double2(fma(-IK, Aw.x, f.x), fma(-IK, Aw.y, f.y));
         Q[node_of<V>(d, i, j)] = from_d2<V>(r64);
         a64x.add(r64.x, r64.x);
         a64y.add(r64.y, r64.y);
@@ -416,7 +418,7 @@ __device__ void refine_tile_fp64(const Ctx& c, int tile, int b, const RState& s,
         c.partS[2 * (int64_t)tile] = sx;
         c.partS[2 * (int64_t)tile + 1] = sy;
     }
-    finish_S(c, b, s, true);
+    finish_S(c, b, s, true, 1.0);
 }
 
 template <typename V, int SCHEME>
@@ -438,7 +440,8 @@ __device__ __forceinline__ void refine_tile(const Ctx& c, int tile, int b, const
 template <typename V, int SCHEME, int LOG2N>
 __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, const RState& s,
                                              const RDesc& d, double* red,
-                                             typename ScalarOf<V>::T* bsc, unsigned* fxs) {
+                                             typename ScalarOf<V>::T* bsc, unsigned* fxs,
+                                             double* rowtab) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const Sz<LOG2N> z(d.log2n);
     const int n = z.n;
@@ -462,6 +465,7 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
         else if (k >= 128 && k < 128 + TR + 2)
             prefetch_l2(static_cast<const V*>(c.T) + node_at(d, z, (r0 - 1 + k - 128) & (n - 1), 0), rb);
     }
+    if (sizeof(V) == 16 && !c.cs.coef) fill_row_table<SCHEME>(rowtab, d.a_matrix, d.a_incl);
     // scalars of this step, converted once (thread 0) to the vector type
     if (threadIdx.x == 0) {
         bsc[0] = (T)s.beta[0];
@@ -552,10 +556,48 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
         w.m0 = d0; w.m1 = d1; w.m2 = d2;
         w.cmm = c0m; w.cm0 = c00;
     };
+    // FP64: rows q0 .. q1 of column j by the weights (StencilRow)
+    auto column64 = [&](int j, int q0, int q1) {
+        if constexpr (sizeof(V) == 16) {
+        const int jm = (j - 1) & (n - 1), jp = (j + 1) & (n - 1);
+        const int pm = pidx(jm), p0 = pidx(j), pp = pidx(jp);
+        const V* up = Pt + (q0 - 1) * SEQ;
+        const V* md = up + SEQ;
+        V u0 = up[pm], u1 = up[p0], u2 = up[pp], m0 = md[pm], m1 = md[p0], m2 = md[pp];
+        // stored scaled by K (row_scale): alpha takes it out (finish_S)
+        auto row = [&](const StencilRow& w, int q, auto doubled) {
+            const V* dn = Pt + (q + 1) * SEQ;
+            const V d0 = dn[pm], d1 = dn[p0], d2 = dn[pp];
+            const V qv = apply_row<SCHEME, decltype(doubled)::value>(w, u0, u1, u2, m0, m1, m2, d0, d1, d2);
+            Q[node_at(d, z, r0 + q - 1, j)] = qv;
+            ax.add(m1.x, qv.x);
+            ay.add(m1.y, qv.y);
+            u0 = m0; u1 = m1; u2 = m2;
+            m0 = d0; m1 = d1; m2 = d2;
+        };
+        if (tc.mrows) {
+            auto bits = [&](int mrow) -> unsigned {   // cells (.., j-1), (.., j)
+                const uint32_t* r = mrows + mrow * wpr;
+                return ((r[jm >> 5] >> (jm & 31)) & 1u) | (((r[j >> 5] >> (j & 31)) & 1u) << 1);
+            };
+            unsigned top = bits(q0 - 1);
+            for (int q = q0; q <= q1; ++q) {
+                const unsigned bot = bits(q);
+                row(table_row<SCHEME>(rowtab, top | (bot << 2)), q, std::true_type());
+                top = bot;
+            }
+        } else {
+            RowWalk<SCHEME> walk(tc.cell(c.cs, d, 0, r0 + q0 - 2, jm), tc.cell(c.cs, d, 0, r0 + q0 - 2, j));
+            for (int q = q0; q <= q1; ++q)
+                row(walk.step(tc.cell(c.cs, d, 0, r0 + q - 1, jm), tc.cell(c.cs, d, 0, r0 + q - 1, j)), q,
+                    std::false_type());
+        }
+        }
+    };
     // n < 256: 256 / n groups of threads share the tile's rows (at n = 64 the
     // columns alone kept 64 of 256 threads busy)
     auto stencil_rows = [&]() {
-        constexpr bool TWO = LOG2N >= 9;   // n >= 512 = 2 x 256 threads
+        constexpr bool TWO = sizeof(V) == 8 && LOG2N >= 9;   // n >= 512 = 2 x 256 threads
         constexpr int W = LOG2N < 8 ? 1 << LOG2N : 256;
         int q0 = 1, q1 = TR;
         if (W < 256) {
@@ -565,6 +607,10 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
             if (q0 > q1) return;
         }
         for (int j = threadIdx.x & (W - 1); j < n; j += TWO ? 512 : 256) {
+            if constexpr (sizeof(V) == 16) {
+                column64(j, q0, q1);
+                continue;
+            }
             Win wa, wb;
             win_start(wa, j, q0);
             if (TWO) win_start(wb, j + 256, q0);
@@ -646,7 +692,7 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
         c.partS[2 * (int64_t)tile] = sx;
         c.partS[2 * (int64_t)tile + 1] = sy;
     }
-    finish_S(c, b, s, false);
+    finish_S(c, b, s, false, sizeof(V) == 16 ? row_scale<SCHEME>() : 1.0);
 }
 
 // The refine or the stencil tile, by the realization's phase (`which`: 1
@@ -657,6 +703,7 @@ __device__ void fused_RS_tile(const Ctx& c, int tile, int which) {
     __shared__ double red[64];   // block_sum2 scratch
     __shared__ unsigned fxs[8];  // row teams' reductions
     __shared__ typename ScalarOf<V>::T bsc[6];
+    __shared__ __align__(16) double rowtab[sizeof(V) == 16 ? ROW_TABLE : 2];   // FP64: stencil rows
     const int b = find_real(c.startS, c.batch, tile);
     const RState& s = c.st[b];
     if (s.phase == PH_DONE || !(which & (s.phase == PH_REFINE ? DO_REFINE : DO_STENCIL))) return;
@@ -665,7 +712,7 @@ __device__ void fused_RS_tile(const Ctx& c, int tile, int which) {
         refine_tile<V, SCHEME>(c, tile, b, s, d);
         return;
     }
-    dispatch_size(d.log2n, [&]<int LG>() { fused_S_body<V, SCHEME, LG>(c, tile, b, s, d, red, bsc, fxs); });
+    dispatch_size(d.log2n, [&]<int LG>() { fused_S_body<V, SCHEME, LG>(c, tile, b, s, d, red, bsc, fxs, rowtab); });
 }
 
 // ----------------------------------------------------------- U kernel --
@@ -916,7 +963,7 @@ inline __device__ void control_apply(const Ctx& c, int b, double pU, double pC) 
     const unsigned upto = k < 2 ? (2u << k) - 1u : 0u;   // correctors 0 .. k
     if (s.phase == PH_ITER) {
         const bool act = mine && s.active[k];
-        const double alpha = act ? c.uscal[4 * b + k] : 0.0;
+        const double alpha = act ? c.uscal[4 * b + 2 + k] : 0.0;
         const double rn = act ? sqrt(pU) : 0.0;
         const unsigned nan = __ballot_sync(0xffffffffu, act && (bad(alpha) || bad(rn) || bad(pC)));
         bool go = false, last = false;
