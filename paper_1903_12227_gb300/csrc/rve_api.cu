@@ -53,43 +53,34 @@ rve_solve_opts resolved_opts(const rve_solve_opts* o) {
 // rows; the stencil tile keeps tS + 2 padded rows in shared memory; column
 // blocks use blockC threads, n / col_seg_rows per column.
 //
-// The heights follow from the nodes of the whole batch.  A block costs a
-// fixed latency and its groups' work, and a pass the blocks of its busiest
-// SM: cost = waves (lat + groups), waves = blocks / slots and half a wave of
-// tail, one at least.  Large batches get the tallest tiles (the halo rows are
-// transformed twice), a single small realization tiles of a few rows, so
-// that all SMs take part: one 32^2 realization in FP64 ran on one SM.
-static double pass_cost(double blocks, double slots, double lat, double groups) {
-    const double x = blocks / slots;
-    return (x > 1.0 ? x + 0.5 : 1.0) * (lat + groups);
-}
-
-static void default_tiles(int n, size_t vb, int blockC, int64_t total, const rve_solve_opts& o, Tiles& t) {
+// The geometry follows from the grid size and the precision alone, never from
+// the rest of the batch: the dot products are summed tile by tile, so a
+// realization's result is the same bits alone and in any batch.  Stencil
+// tiles: the height with the least ceil(n / tS) blocks times a block's latency
+// and transform groups (the halo rows are transformed twice); FP64, bound by
+// arithmetic, the lower of two within 15 %, so that few realizations spread
+// over more SMs.
+static void default_tiles(int n, size_t vb, int blockC, const rve_solve_opts& o, Tiles& t) {
     const size_t seq = (size_t)seq_stride(n);
     const int G = std::max(1, 2048 / n);
-    const double rows_all = (double)total / (double)n;   // of the batch, were it all of size n
-    // latency in units of a transform group's work (FP64 groups are heavier)
-    const double lat = vb == 8 ? 0.7 : 0.2;
-    const double slotsS = 152.0 * (vb == 8 ? 3 : 2), slotsU = 152.0 * (vb == 8 ? 4 : 2);
-    // update blocks: up to U_GROUPS groups streamed; parts of a group on grids
-    // of many rows per group
-    t.tU = std::min(n, G);
-    double best = 1e300;
-    for (int r = std::min(n, U_GROUPS * G); r >= std::max(1, std::min(G, 4)); r /= 2) {
-        const double cost = pass_cost(rows_all / r, slotsU, lat, (double)r / G);
-        if (cost < best) { best = cost; t.tU = r; }
-    }
-    // stencil tiles: tS + 2 a multiple of G (no idle row slots), a part of G,
-    // or the whole realization (no halo) where it fits; within ~72 KB (three
-    // blocks per SM), or 110 KB on grids whose rows leave fewer than four
+    // update blocks: mixed, U_GROUPS groups, each streamed in while the one
+    // before it transforms; FP64, bound by arithmetic, fewer rows on more SMs
+    t.tU = std::min(n, vb == 8 ? U_GROUPS * G : (n <= 256 ? G : 2 * G));
+    // stencil tiles: tS + 2 a multiple of G (no idle row slots), or the whole
+    // realization (no halo) up to n = 64; within ~72 KB (three blocks per SM),
+    // or 110 KB on grids whose rows leave fewer than four
     auto smem_of = [&](int ts) {
         return (size_t)(ts + 2) * seq * vb + (size_t)(ts + 1) * (n / 32) * 4;
     };
-    t.tS = 0;
-    best = 1e300;
+    const double lat = vb == 8 ? 0.7 : 0.2;   // in units of a group's work (FP64 groups are heavier)
+    t.tS = 1;
+    double best = 1e300;
     auto consider = [&](int ts, int transformed) {
-        const double cost = pass_cost(rows_all / ts, slotsS, lat, (double)transformed / G);
-        if (cost < best) { best = cost; t.tS = ts; }
+        const double cost = ((n + ts - 1) / ts) * (lat + (double)transformed / G);
+        if (cost < (vb == 16 && ts < t.tS ? 1.15 : 1.0) * best) {
+            best = std::min(best, cost);
+            t.tS = ts;
+        }
     };
     for (size_t budget : {(size_t)73728, (size_t)112640}) {
         if (n <= 64 && smem_of(n) <= budget) consider(n, n);
@@ -97,11 +88,8 @@ static void default_tiles(int n, size_t vb, int blockC, int64_t total, const rve
             const int ts = k * G - 2;
             if (ts >= 1 && ts < n && smem_of(ts) <= budget) consider(ts, ts + 2);
         }
-        for (int g = G / 2; g >= 4; g /= 2)
-            if (g - 2 < n && smem_of(g - 2) <= budget) consider(g - 2, g);
         if (smem_of(4) <= budget) break;   // else: large grids, fewer and taller tiles
     }
-    if (t.tS < 1) t.tS = 1;
     int ts_tuned = 0, bc_tuned = 0;
     if (tuned_tiles(n, o.precision, o.path == RVE_PATH_PERSISTENT ? 1 : 0, &ts_tuned, &bc_tuned))
         t.tS = ts_tuned;
@@ -137,28 +125,19 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
     p.words = 0;
     p.max_log2n = 5;
     p.smemS = p.smemU = p.smemC = 0;
-    int64_t maxnb = 0, total = 0, colthreads = 0;
+    int64_t maxnb = 0;
     int maxn = 0;
     for (int b = 0; b < batch; ++b) {
         const int64_t nn = (int64_t)r[b].L * r[b].m0;
         if (nn < MIN_N || nn > MAX_N) continue;   // rejected below
         maxn = std::max(maxn, (int)nn);
-        total += nn * nn;
-        colthreads += nn * (nn / col_seg_rows((int)nn, (int)p.vbytes));
     }
     // column blocks: a segment of up to 32 rows per thread in registers.
     // Mixed: 128 threads (3 % faster than 256 and 13 % faster than 512 on
     // 512^2 grids, measured), more where 128 would leave a block under eight
-    // columns, whose rows are its memory accesses.  FP64: 256 threads, two
-    // blocks per SM
-    p.blockC = (p.vbytes == 8) ? (maxn > 1024 ? 512 : maxn > 512 ? 256 : 128) : 256;
-    // few columns in all: smaller blocks on more SMs, at least four (FP64:
-    // two) columns of the largest grid each
-    {
-        const int segs = std::max(1, maxn / col_seg_rows(std::max(maxn, MIN_N), (int)p.vbytes));
-        const int least = std::max(64, segs * (p.vbytes == 8 ? 4 : 2));
-        while (colthreads < (int64_t)p.blockC * 304 && p.blockC / 2 >= least) p.blockC /= 2;
-    }
+    // columns, whose rows are its memory accesses.  FP64: 128 threads (1024^2:
+    // 47 us a pass, 51 us at 256), at least two columns
+    p.blockC = (p.vbytes == 8) ? (maxn > 1024 ? 512 : maxn > 512 ? 256 : 128) : (maxn > 1024 ? 256 : 128);
     {
         int ts_tuned = 0, bc_tuned = 0;
         if (maxn > 0 && tuned_tiles(maxn, o.precision, o.path == RVE_PATH_PERSISTENT ? 1 : 0,
@@ -180,7 +159,7 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
             !(x.a_incl > 0.0))
             return RVE_EINVAL;
         Tiles t;
-        default_tiles(n, p.vbytes, p.blockC, total, o, t);
+        default_tiles(n, p.vbytes, p.blockC, o, t);
         const int segs = n / col_seg_rows(n, (int)p.vbytes);   // threads per column
         if (t.tS < 1 || t.tS > n || t.tC < 1 || !pow2(t.tC) || n % t.tC ||
             t.tC * segs > p.blockC)

@@ -1,7 +1,5 @@
-"""Tile heights follow from the batch's size: solves of one realization, of a
-few and of many, over the grid sizes where whole tiles, row groups and parts of
-a transform group meet, against each other and the true residual."""
-import numpy as np
+"""Stencil tiles, whole-realization tiles and row groups over the grid sizes: the
+true residual of batched solves, and a lone solve against the batch bit for bit."""
 import pytest
 import torch
 
@@ -26,10 +24,8 @@ def test_lone_and_batched_solves(n, count, scheme, precision):
     # A u (8 eps |A| |u| per node, |A| <= 16 a_max) and, mixed, of the final u
     floor = 64 * 2.0 ** -53 * 160.0 * u.view(count, -1, 2).abs().amax(1) * n
     assert bool((r.norm(dim=1) <= tol * f.view(count, n * n, 2).norm(dim=1) + floor).all())
-    A = rve.a_hom(ds, u, mask=mask, scheme=scheme)
     words = n * n // 32
-    for k in (0, count - 1):   # two answers to the same tolerance: the energies differ by its square
+    for k in (0, count - 1):
         m = mask[k * words:(k + 1) * words]
         v, _ = rve.solve(ds[k:k + 1], mask=m, opts=opts)
-        B = rve.a_hom(ds[k:k + 1], v, mask=m, scheme=scheme)
-        np.testing.assert_allclose(B[0].cpu().numpy(), A[k].cpu().numpy(), rtol=0, atol=1e-10)
+        assert torch.equal(v, u[k * n * n:(k + 1) * n * n])
