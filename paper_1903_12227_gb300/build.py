@@ -48,7 +48,7 @@ def _compile(src: str, extra: list) -> str:
     obj = os.path.join(BUILD_DIR, os.path.splitext(src)[0] + ".o")
     # the pipeline's size dispatch uses templated lambdas (C++20); the other
     # units stay C++17
-    std = "-std=c++20" if src.startswith(("rve_solver", "rve_pipe", "rve_persist")) else "-std=c++17"
+    std = "-std=c++20" if src.startswith(("rve_solver", "rve_pipe", "rve_persist", "rve_ops")) else "-std=c++17"
     cmd = [nvcc(), *ARCH, "-O3", "-lineinfo", std, "-Xcompiler", "-fPIC",
            "-I", INCLUDE, "-I", CSRC, "-c", os.path.join(CSRC, src), "-o", obj, *extra]
     r = subprocess.run(cmd, capture_output=True, text=True)

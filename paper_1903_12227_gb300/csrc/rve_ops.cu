@@ -1,8 +1,10 @@
 // rve_ops.cu -- field generation, right-hand sides, stiffness apply,
 // homogenized matrix and its adjoint (sm_103a).
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "rve_ahom.cuh"
 #include "rve_common.cuh"
@@ -76,18 +78,137 @@ __device__ __forceinline__ V ldv(const V* __restrict__ x, const RDesc& d, int i,
     return x[d.node_off + ((int64_t)(i & (d.n - 1)) << d.log2n) + (j & (d.n - 1))];
 }
 
+// y = A x.  A thread walks down `rows` rows of one column (FP64) or two (FP32)
+// with the 3 x 3 neighbourhood in registers, so that a node costs the loads of
+// its row's new neighbours; 256 threads take min(n, 256) columns (FP32: min(n,
+// 512)) and, on smaller grids, several groups of rows.  FP32: the cell values
+// stay in FP32 -- through double, as the cell accessor returns them, every node
+// cost four conversions on the FP64 pipe -- and the kernel is bound by memory:
+// 96 x 512^2 nodes 250 -> 96 us.  FP64: bound by the FP64 pipe (StencilRow);
+// 11 x 1024^2 nodes, explicit cells 629 -> 570 us.
+constexpr int STIFF_THREADS = 256;
+template <typename V> __host__ __device__ constexpr int stiff_cols(int n) {   // columns of a block
+    return n < (int)(4096 / sizeof(V)) ? n : (int)(4096 / sizeof(V));
+}
+// Rows of a block: `rows` per thread and group.
+template <typename V> __host__ __device__ constexpr int stiff_block_rows(int n, int rows) {
+    const int groups = STIFF_THREADS / (stiff_cols<V>(n) / (int)(16 / sizeof(V)));
+    return groups * rows < n ? groups * rows : n;
+}
+
 template <int SCHEME, typename V>
-__global__ void k_stiffness(const __grid_constant__ DescChunk ch, CoefSrc cs,
-                            const V* __restrict__ x, V* __restrict__ y) {
+__global__ void __launch_bounds__(STIFF_THREADS) k_stiffness(const __grid_constant__ DescChunk ch,
+                                                             CoefSrc cs, const V* __restrict__ x,
+                                                             V* __restrict__ y, int rows,
+                                                             bool pairs) {
+    __shared__ __align__(16) double rowtab[sizeof(V) == 16 ? ROW_TABLE : 2];
     const int b = find_real(ch.start, ch.count, blockIdx.x);
     const RDesc& d = ch.d[b];
-    const int64_t node = (int64_t)(blockIdx.x - ch.start[b]) * NODE_TILE + threadIdx.x;
-    const int i = (int)(node >> d.log2n), j = (int)(node & (d.n - 1));
-    const CellsT<typename ScalarOf<V>::T> a = cells_as<typename ScalarOf<V>::T>(cells_at(cs, d, i, j));
-    y[d.node_off + node] = stencil_apply<SCHEME, V>(
-        a, ldv(x, d, i - 1, j - 1), ldv(x, d, i - 1, j), ldv(x, d, i - 1, j + 1),
-        ldv(x, d, i, j - 1), ldv(x, d, i, j), ldv(x, d, i, j + 1),
-        ldv(x, d, i + 1, j - 1), ldv(x, d, i + 1, j), ldv(x, d, i + 1, j + 1));
+    const int n = d.n, m = n - 1, lg = d.log2n;
+    constexpr int CPT = 16 / sizeof(V);                     // columns of a thread
+    const int CW = stiff_cols<V>(n), BR = stiff_block_rows<V>(n, rows);
+    const int across = CW / CPT, groups = STIFF_THREADS / across;
+    const int per = (BR + groups - 1) / groups;             // rows of a thread
+    const int blk = blockIdx.x - ch.start[b], cblks = n / CW;
+    const int g = threadIdx.x / across;
+    const int j = (blk % cblks) * CW + CPT * (threadIdx.x - g * across);
+    const int i0 = (blk / cblks) * BR + g * per, i1 = min(i0 + per, (blk / cblks) * BR + BR);
+    const V* __restrict__ xb = x + d.node_off;
+    V* __restrict__ yb = y + d.node_off;
+    const uint32_t* __restrict__ mw = cs.coef ? nullptr : cs.mask + d.word_off;
+    const double* __restrict__ cf = cs.coef ? cs.coef + d.node_off : nullptr;
+    const int jm = (j - 1) & m, jp = (j + CPT) & m;
+    // bits of cells (i, j - 1), (i, j), (i, j + 1) (j even for FP32, so the last two share a word)
+    auto bits = [&](int i) -> unsigned {
+        const int64_t r = (int64_t)(i & m) << lg;
+        const uint32_t w = __ldg(mw + ((r + j) >> 5)) >> (j & 31);
+        const uint32_t v = (j & 31) ? __ldg(mw + ((r + j) >> 5)) >> ((j & 31) - 1)
+                                    : __ldg(mw + ((r + jm) >> 5)) >> 31;
+        return (v & 1u) | ((w & 3u) << 1);
+    };
+    if constexpr (sizeof(V) == 16) {
+        if (mw) {
+            fill_row_table<SCHEME>(rowtab, d.a_matrix, d.a_incl);
+            __syncthreads();
+        }
+        if (i0 >= i1) return;
+        auto at = [&](int i, int jj) { return __ldg(xb + ((int64_t)(i & m) << lg) + jj); };
+        V u0 = at(i0 - 1, jm), u1 = at(i0 - 1, j), u2 = at(i0 - 1, jp);
+        V m0 = at(i0, jm), m1 = at(i0, j), m2 = at(i0, jp);
+        auto row = [&](const StencilRow& w, int i, const V& d0, const V& d1, const V& d2, auto doubled) {
+            constexpr double IK = 1.0 / row_scale<SCHEME>();
+            const V q = apply_row<SCHEME, decltype(doubled)::value>(w, u0, u1, u2, m0, m1, m2, d0, d1, d2);
+            yb[((int64_t)i << lg) + j] = make_double2(IK * q.x, IK * q.y);
+            u0 = m0; u1 = m1; u2 = m2;
+            m0 = d0; m1 = d1; m2 = d2;
+        };
+        if (mw) {
+            unsigned top = bits(i0 - 1) & 3u;
+#pragma unroll 2
+            for (int i = i0; i < i1; ++i) {
+                const V d0 = at(i + 1, jm), d1 = at(i + 1, j), d2 = at(i + 1, jp);
+                const unsigned bot = bits(i) & 3u;
+                row(table_row<SCHEME>(rowtab, top | (bot << 2)), i, d0, d1, d2, std::true_type());
+                top = bot;
+            }
+        } else {
+            auto cell = [&](int i, int jj) { return __ldg(cf + ((int64_t)(i & m) << lg) + jj); };
+            RowWalk<SCHEME> walk(cell(i0 - 1, jm), cell(i0 - 1, j));
+#pragma unroll 2
+            for (int i = i0; i < i1; ++i) {
+                const V d0 = at(i + 1, jm), d1 = at(i + 1, j), d2 = at(i + 1, jp);
+                row(walk.step(cell(i, jm), cell(i, j)), i, d0, d1, d2, std::false_type());
+            }
+        }
+    } else {
+        if (i0 >= i1) return;
+        const float ai = (float)d.a_incl, am = (float)d.a_matrix;
+        struct Row { V l, a, b, r; };     // x at j - 1, j, j + 1, j + 2
+        struct Cel { float l, a, b; };    // cells j - 1, j, j + 1
+        // `pairs`: x and y are 16-byte aligned (the ABI asks for 8)
+        auto xrow = [&](int i) -> Row {
+            const V* p = xb + ((int64_t)(i & m) << lg);
+            float4 c;
+            if (pairs) {
+                c = __ldg(reinterpret_cast<const float4*>(p + j));
+            } else {
+                const V a = __ldg(p + j), b2 = __ldg(p + j + 1);
+                c = make_float4(a.x, a.y, b2.x, b2.y);
+            }
+            return Row{__ldg(p + jm), make_float2(c.x, c.y), make_float2(c.z, c.w), __ldg(p + jp)};
+        };
+        auto crow = [&](int i) -> Cel {
+            if (mw) {
+                const unsigned k = bits(i);
+                return Cel{(k & 1u) ? ai : am, (k & 2u) ? ai : am, (k & 4u) ? ai : am};
+            }
+            const double* p = cf + ((int64_t)(i & m) << lg);
+            return Cel{(float)__ldg(p + jm), (float)__ldg(p + j), (float)__ldg(p + j + 1)};
+        };
+        Row u = xrow(i0 - 1), c = xrow(i0), ahead = xrow(i0 + 1);   // one row ahead of its use
+        Cel t = crow(i0 - 1), o = crow(i0);
+#pragma unroll 4
+        for (int i = i0; i < i1; ++i) {
+            const Row dn = ahead;
+            ahead = xrow(i + 2);
+            const Cel on = crow(i + 1);
+            const V q0 = stencil_apply<SCHEME, V>(CellsT<float>{t.l, t.a, o.l, o.a}, u.l, u.a, u.b, c.l, c.a,
+                                                  c.b, dn.l, dn.a, dn.b);
+            const V q1 = stencil_apply<SCHEME, V>(CellsT<float>{t.a, t.b, o.a, o.b}, u.a, u.b, u.r, c.a, c.b,
+                                                  c.r, dn.a, dn.b, dn.r);
+            V* o2 = yb + ((int64_t)i << lg) + j;
+            if (pairs) {
+                *reinterpret_cast<float4*>(o2) = make_float4(q0.x, q0.y, q1.x, q1.y);
+            } else {
+                o2[0] = q0;
+                o2[1] = q1;
+            }
+            u = c;
+            c = dn;
+            t = o;
+            o = on;
+        }
+    }
 }
 
 // y = M x, M = M1 (x) M1 the Q1 mass matrix (1D: consistent h [1/6, 2/3,
@@ -154,6 +275,130 @@ __global__ void __launch_bounds__(NODE_TILE) k_cheb(const __grid_constant__ Desc
     for (int k = 0; k < 4; ++k) {
         const double sum = block_sum(v[k], red);
         if (threadIdx.x == 0) part[(int64_t)blockIdx.x * 4 + k] = sum;
+    }
+}
+
+// The whole recurrence of a realization of n <= 128 in one cluster of eight
+// blocks: block r keeps its n / 8 rows of w_k and w_{k-1} in shared memory and
+// reads the rows next to them from its neighbours' (distributed shared
+// memory); one cluster barrier per step, behind which w_{k-1} may be
+// overwritten (only w_k is read by others).  No step waits for its sums: the
+// threads leave them in shared memory, the ninth warp adds them up during the
+// next step and block 0's forms the moments in the one after.  As two launches
+// per step, 16 realizations of 64^2 took 18 us a step, 4 of them work: 4725 ->
+// 1655 us for 512 moments; now bound by the FP64 pipe (18 operations per node
+// and step, lumped) and the barrier.
+constexpr int CHEB_CTAS = 8, CHEB_WARPS = 8, CHEB_MAX_N = 128;
+template <int SCHEME>
+__global__ void __cluster_dims__(CHEB_CTAS, 1, 1) __launch_bounds__(32 * (CHEB_WARPS + 1))
+    k_cheb_cluster(const __grid_constant__ DescChunk ch, CoefSrc cs, double a0, double a1, int steps,
+                   int K, const double* __restrict__ v, double* __restrict__ mu) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ __align__(16) double rowtab[ROW_TABLE];
+    __shared__ __align__(16) double psum[2][32 * CHEB_WARPS * 4];   // the threads' sums, by step parity
+    __shared__ double slots[2][CHEB_CTAS * 4];   // block 0: the blocks' sums, by step parity
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int rank = (int)cl.block_rank(), b = blockIdx.x / CHEB_CTAS;
+    const RDesc& d = ch.d[b];
+    const int n = d.n, m = n - 1, lg = d.log2n, R = n / CHEB_CTAS, r0 = rank * R;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int rows = R * n;
+    double2* own = reinterpret_cast<double2*>(smem_raw);   // [2][R][n]
+    const double2* above = cl.map_shared_rank(own, (rank + CHEB_CTAS - 1) % CHEB_CTAS) + (R - 1) * n;
+    const double2* below = cl.map_shared_rank(own, (rank + 1) % CHEB_CTAS);
+    double* slot0 = cl.map_shared_rank(&slots[0][0], 0);
+    for (int k = tid; k < rows; k += blockDim.x) {   // v is 8-byte aligned
+        const int64_t i = 2 * (d.node_off + (int64_t)r0 * n + k);
+        own[k] = make_double2(v[i], v[i + 1]);
+    }
+    const bool masked = !cs.coef;
+    if (masked) fill_row_table<SCHEME>(rowtab, d.a_matrix, d.a_incl);
+    // column j, rows i0 .. i1 of the block
+    const int groups = 32 * CHEB_WARPS / n, per = max(1, R / groups);
+    const int j = tid & m, jm = (j - 1) & m, jp = (j + 1) & m;
+    const int i0 = (tid >> lg) * per, i1 = min(R, i0 + per);
+    const bool active = tid < 32 * CHEB_WARPS && i0 < R;
+    auto cell = [&](int i, int jj) { return cs.cell(d, (r0 + i) & m, jj); };
+    unsigned pat = 0;   // masks: two bits per row i0 - 1 .. i1 - 1 (at most nine rows)
+    if (active && masked) {
+        const uint32_t* mw = cs.mask + d.word_off;
+        for (int i = i0 - 1; i < i1; ++i) {
+            const int64_t r = (int64_t)((r0 + i) & m) << lg;
+            const unsigned x = (mw[(r + jm) >> 5] >> (jm & 31)) & 1u, y = (mw[(r + j) >> 5] >> (j & 31)) & 1u;
+            pat |= (x | (y << 1)) << (2 * (i - i0 + 1));
+        }
+    }
+    double mu0 = 0.0, mu1 = 0.0;   // block 0, ninth warp: the first moments
+    cl.sync();
+    const int summers = n * (R / per);   // threads that hold sums: a multiple of 8
+    for (int k = 0; k < steps + 2; ++k) {
+        const int cur = (k & 1) * rows, oth = rows - cur;
+        if (active && k < steps) {
+            double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+            const double f = k == 0 ? 1.0 : 2.0;
+            const double f1 = f * a0 / row_scale<SCHEME>(), f2 = f * a1;
+            auto rowp = [&](int i) -> const double2* {
+                return i < 0 ? above + cur : i >= R ? below + cur : own + cur + i * n;
+            };
+            const double2* up = rowp(i0 - 1);
+            const double2* md = rowp(i0);
+            double2 u0 = up[jm], u1 = up[j], u2 = up[jp], c0 = md[jm], c1 = md[j], c2 = md[jp];
+            auto row = [&](int i, const StencilRow& w, auto doubled) {
+                const double2* dn = rowp(i + 1);
+                const double2 d0 = dn[jm], d1 = dn[j], d2 = dn[jp];
+                const double2 q = apply_row<SCHEME, decltype(doubled)::value>(w, u0, u1, u2, c0, c1, c2, d0, d1, d2);
+                const double2 wm = k == 0 ? make_double2(0.0, 0.0) : own[oth + i * n + j];
+                const double2 t = make_double2(fma(f1, q.x, fma(-f2, c1.x, -wm.x)),
+                                               fma(f1, q.y, fma(-f2, c1.y, -wm.y)));
+                own[oth + i * n + j] = t;
+                s0 = fma(c1.x, c1.x, s0);
+                s1 = fma(c1.y, c1.y, s1);
+                s2 = fma(t.x, c1.x, s2);
+                s3 = fma(t.y, c1.y, s3);
+                u0 = c0; u1 = c1; u2 = c2;
+                c0 = d0; c1 = d1; c2 = d2;
+            };
+            if (masked) {
+                for (int i = i0; i < i1; ++i)
+                    row(i, table_row<SCHEME>(rowtab, (pat >> (2 * (i - i0))) & 15u), std::true_type());
+            } else {
+                RowWalk<SCHEME> walk(cell(i0 - 1, jm), cell(i0 - 1, j));
+                for (int i = i0; i < i1; ++i) row(i, walk.step(cell(i, jm), cell(i, j)), std::false_type());
+            }
+            double2* ps = reinterpret_cast<double2*>(psum[k & 1]) + 2 * tid;
+            ps[0] = make_double2(s0, s1);
+            ps[1] = make_double2(s2, s3);
+        }
+        if (tid >= 32 * CHEB_WARPS) {
+            // w.w (0, 1) and w'.w (2, 3) of the block, in lanes value, value + 4, ...
+            if (k >= 1 && k - 1 < steps) {
+                const double* ps = psum[(k - 1) & 1] + lane;
+                double x = 0.0, y = 0.0;
+                for (int t = 0; t + 16 <= summers; t += 16) {
+                    x += ps[4 * t];
+                    y += ps[4 * t + 32];
+                }
+                x += y;
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                if (lane < 4) slot0[((k - 1) & 1) * CHEB_CTAS * 4 + rank * 4 + lane] = x;
+            }
+            if (rank == 0 && k >= 2) {
+                const int q = k - 2;
+                double x = slots[q & 1][lane];
+#pragma unroll
+                for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                const double nc = __shfl_down_sync(0xffffffffu, x, 2);   // lanes 0, 1
+                if (lane < 2) {
+                    double* mb = mu + ((int64_t)b * 2 + lane) * K;
+                    if (q == 0) { mu0 = x; mu1 = nc; }
+                    if (2 * q < K) mb[2 * q] = q == 0 ? x : 2.0 * x - mu0;
+                    if (2 * q + 1 < K) mb[2 * q + 1] = q == 0 ? nc : 2.0 * nc - mu1;
+                }
+            }
+        }
+        cl.sync();
     }
 }
 
@@ -325,21 +570,25 @@ cudaError_t launch_coef_from_mask(const Plan& p, const uint32_t* mask, double* c
 cudaError_t launch_stiffness(const Plan& p, void*, const uint32_t* mask, const double* coef,
                              int scheme, int precision, const void* x, void* y, cudaStream_t s) {
     CoefSrc cs{mask, coef};
-    return for_chunks(p, node_tiles, [&](const DescChunk& ch, int) {
-        const int g = ch.start[ch.count];
-        if (precision == RVE_FP64) {
-            const double2* xx = static_cast<const double2*>(x);
-            double2* yy = static_cast<double2*>(y);
-            if (scheme == RVE_Q1_LUMPED) k_stiffness<1, double2><<<g, NODE_TILE, 0, s>>>(ch, cs, xx, yy);
-            else k_stiffness<0, double2><<<g, NODE_TILE, 0, s>>>(ch, cs, xx, yy);
-        } else {
-            const float2* xx = static_cast<const float2*>(x);
-            float2* yy = static_cast<float2*>(y);
-            if (scheme == RVE_Q1_LUMPED) k_stiffness<1, float2><<<g, NODE_TILE, 0, s>>>(ch, cs, xx, yy);
-            else k_stiffness<0, float2><<<g, NODE_TILE, 0, s>>>(ch, cs, xx, yy);
-        }
-        return cudaGetLastError();
-    });
+    // rows per thread: 16, fewer while that leaves under four blocks per SM
+    auto launch = [&]<typename V>(const V* xx, V* yy) {
+        const bool pairs = ((reinterpret_cast<uintptr_t>(xx) | reinterpret_cast<uintptr_t>(yy)) & 15) == 0;
+        int rows = 16;
+        while (rows > 2 && p.nodes < (int64_t)rows * STIFF_THREADS * (int64_t)(16 / sizeof(V)) * 4 * 152) rows /= 2;
+        return for_chunks(p,
+                          [&](const RDesc& d) {
+                              return (int64_t)(d.n / stiff_cols<V>(d.n)) * (d.n / stiff_block_rows<V>(d.n, rows));
+                          },
+                          [&](const DescChunk& ch, int) {
+                              const int g = ch.start[ch.count];
+                              if (scheme == RVE_Q1_LUMPED) k_stiffness<1, V><<<g, STIFF_THREADS, 0, s>>>(ch, cs, xx, yy, rows, pairs);
+                              else k_stiffness<0, V><<<g, STIFF_THREADS, 0, s>>>(ch, cs, xx, yy, rows, pairs);
+                              return cudaGetLastError();
+                          });
+    };
+    if (precision == RVE_FP64)
+        return launch(static_cast<const double2*>(x), static_cast<double2*>(y));
+    return launch(static_cast<const float2*>(x), static_cast<float2*>(y));
 }
 
 cudaError_t launch_mass(const Plan& p, int scheme, const double* x, double* y, cudaStream_t s) {
@@ -373,15 +622,32 @@ cudaError_t launch_cheb(const Plan& p, void* ws, const uint32_t* mask, const dou
     double2* wa = reinterpret_cast<double2*>(w);
     double2* wb = reinterpret_cast<double2*>(w + up(sizeof(double2) * (size_t)p.nodes));
     double* part = reinterpret_cast<double*>(w + 2 * up(sizeof(double2) * (size_t)p.nodes));
-    cudaError_t e = cudaMemcpyAsync(wb, v, sizeof(double2) * (size_t)p.nodes,
-                                    cudaMemcpyDeviceToDevice, s);   // w_0
-    if (e != cudaSuccess) return e;
     const double a0 = 2.0 / (hi - lo), a1 = (hi + lo) / (hi - lo);
     CoefSrc cs{mask, coef};
     const int steps = (K + 1) / 2;
+    const size_t most = 2 * sizeof(double2) * CHEB_MAX_N * CHEB_MAX_N / CHEB_CTAS;
+    cudaError_t e = cudaFuncSetAttribute(k_cheb_cluster<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_cheb_cluster<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    if (e != cudaSuccess) return e;
     return for_chunks(p, node_tiles, [&](const DescChunk& ch, int first_real) {
-        const int g = ch.start[ch.count];
         double* m = mu + (int64_t)first_real * 2 * K;
+        int maxn = 0;
+        int64_t nodes = 0;
+        for (int k = 0; k < ch.count; ++k) {
+            maxn = std::max(maxn, ch.d[k].n);
+            nodes += (int64_t)ch.d[k].n * ch.d[k].n;
+        }
+        if (maxn <= CHEB_MAX_N) {   // two vectors of a realization fit a cluster's shared memory
+            const size_t smem = 2 * sizeof(double2) * (size_t)maxn * maxn / CHEB_CTAS;
+            auto kern = scheme == RVE_Q1_LUMPED ? k_cheb_cluster<1> : k_cheb_cluster<0>;
+            kern<<<ch.count * CHEB_CTAS, 32 * (CHEB_WARPS + 1), smem, s>>>(ch, cs, a0, a1, steps, K, v, m);
+            return cudaGetLastError();
+        }
+        const cudaError_t ce = cudaMemcpyAsync(wb + ch.d[0].node_off, v + 2 * ch.d[0].node_off,
+                                               sizeof(double2) * (size_t)nodes, cudaMemcpyDeviceToDevice, s);   // w_0
+        if (ce != cudaSuccess) return ce;
+        const int g = ch.start[ch.count];
         double2* cur = wb;    // w_k
         double2* oth = wa;    // in: w_{k-1}, out: w_{k+1}
         for (int k = 0; k < steps; ++k) {
