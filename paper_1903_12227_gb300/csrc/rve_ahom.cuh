@@ -219,7 +219,100 @@ __device__ __forceinline__ void a_hom_strip(const RDesc& d, int strip, CoefSrc c
     a_hom_block_sums(acc, red, out);
 }
 
-// FP64 form of a_hom_tile (the A_hom of FP64 solves): the same cell sums in
+// The energy form alone in double-double arithmetic (the A_hom of FP64 solves;
+// a_hom_tile_dd below adds the flux form).  FP64 operations are what it costs:
+// differences of u across a cell and the added h are two TwoSums, left
+// unnormalised; the products of a cell are gathered as in a compensated dot
+// product (Ogita, Rump & Oishi's Dot2: TwoProd, TwoSum, the errors added up in
+// a double), and only a thread's sums are normalised.  The error is O(eps^2) of
+// the terms' size, 390 operations per cell instead of 1680; 1024^2 cells 2.81 ->
+// 0.90 ms.  Partials out[2k], out[2k+1] (k = 1, 2, 3) = (hi, lo) of E_11,
+// E_12, E_22, valid in thread 0; `red` holds 32 ddouble (shared).
+struct dd_sum {   // sum of unevaluated (p, c): errors in lo
+    double hi, lo;
+    __device__ __forceinline__ void add(double p, double c) {
+        const ddouble s = dd_two_sum(hi, p);
+        hi = s.hi;
+        lo = __dadd_rn(lo, __dadd_rn(s.lo, c));
+    }
+    // x y of unnormalised pairs
+    __device__ __forceinline__ void add_product(ddouble x, ddouble y) {
+        const double p = __dmul_rn(x.hi, y.hi);
+        add(p, __fma_rn(x.hi, y.lo, __fma_rn(x.lo, y.hi, __fma_rn(x.hi, y.hi, -p))));
+    }
+};
+template <int SCHEME>
+__device__ __forceinline__ void a_hom_tile_energy(const RDesc& d, int64_t tile, int cells, CoefSrc cs,
+                                                  const double2* __restrict__ u, ddouble* red,
+                                                  double* out) {
+    const double h = d.h;
+    const int n = d.n;
+    auto at = [&](int i, int j) {   // periodic node access
+        return u[d.node_off + ((int64_t)(i & (n - 1)) << d.log2n) + (j & (n - 1))];
+    };
+    auto diff = [](double a, double b) { return dd_two_sum(a, -b); };
+    auto diff_h = [](double a, double b, double c) -> ddouble {   // (a - b) + c
+        const ddouble s = dd_two_sum(a, -b), t = dd_two_sum(s.hi, c);
+        return {t.hi, __dadd_rn(s.lo, t.lo)};
+    };
+    dd_sum acc[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
+    for (int t = threadIdx.x; t < cells; t += blockDim.x) {
+        const int64_t cidx = tile * cells + t;
+        const int i = (int)(cidx >> d.log2n), j = (int)(cidx & (n - 1));
+        double a;
+        if (cs.coef) {
+            a = __ldg(cs.coef + d.node_off + cidx);
+        } else {
+            const uint32_t w = __ldg(cs.mask + d.word_off + (cidx >> 5));
+            a = ((w >> (cidx & 31)) & 1u) ? d.a_incl : d.a_matrix;
+        }
+        const double2 r00 = at(i, j), r01 = at(i, j + 1), r10 = at(i + 1, j), r11 = at(i + 1, j + 1);
+        dd_sum e[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
+        // edges and diagonals of the cell, v_i = xi_i + u_i (see a_hom_cell)
+        auto pair = [&](ddouble v1, ddouble v2, double wgt) {
+            const ddouble w1 = dd_scale2(v1, wgt);
+            e[0].add_product(w1, v1);
+            e[1].add_product(w1, v2);
+            e[2].add_product(dd_scale2(v2, wgt), v2);
+        };
+        pair(diff(r01.x, r00.x), diff_h(r01.y, r00.y, h), 1.0);
+        pair(diff_h(r10.x, r00.x, h), diff(r10.y, r00.y), 1.0);
+        pair(diff_h(r11.x, r01.x, h), diff(r11.y, r01.y), 1.0);
+        pair(diff(r11.x, r10.x), diff_h(r11.y, r10.y, h), 1.0);
+        if (SCHEME == 0) {
+            pair(diff_h(r11.x, r00.x, h), diff_h(r11.y, r00.y, h), 2.0);
+            pair(diff_h(r10.x, r01.x, h), diff_h(r10.y, r01.y, -h), 2.0);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) acc[k].add_product(ddouble{e[k].hi, e[k].lo}, ddouble{a, 0.0});
+    }
+    // three sums over the warp in six additions per lane: halves, then quarters
+    // of the warp keep one sum each (lanes 0, 8, 16 end with E_11, E_12, E_22)
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    ddouble v[4];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) v[k] = dd_fast_two_sum(acc[k].hi, acc[k].lo);
+    v[3] = ddouble{0.0, 0.0};
+    auto other = [](ddouble x, int o) -> ddouble {
+        return {__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
+    };
+    const bool h16 = lane & 16, h8 = lane & 8;
+    const ddouble x0 = dd_add(h16 ? v[2] : v[0], other(h16 ? v[0] : v[2], 16));
+    const ddouble x1 = dd_add(h16 ? v[3] : v[1], other(h16 ? v[1] : v[3], 16));
+    ddouble x = dd_add(h8 ? x1 : x0, other(h8 ? x0 : x1, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) x = dd_add(x, other(x, o));
+    if ((lane & 7) == 0) red[wid * 4 + (lane >> 3)] = x;
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        ddouble s = red[threadIdx.x];
+        for (int w = 1; w < nw; ++w) s = dd_add(s, red[w * 4 + threadIdx.x]);
+        out[2 * (threadIdx.x + 1)] = s.hi;
+        out[2 * (threadIdx.x + 1) + 1] = s.lo;
+    }
+}
+
+// FP64 form of a_hom_tile, energy and flux: the same cell sums in
 // double-double arithmetic on the FP64 pipe.  Differences of u across a cell
 // are exact (TwoSum), products and sums carry ~106 bits, so the only error
 // left in A_hom is that of the correctors themselves -- which enters the
@@ -227,7 +320,7 @@ __device__ __forceinline__ void a_hom_strip(const RDesc& d, int strip, CoefSrc c
 // Partials out[2k], out[2k+1] = (hi, lo) of the same eight sums, valid in
 // thread 0; `red` holds 32 * AHOM_NP ddouble (shared).  Contains barriers.
 template <int SCHEME>
-__device__ __forceinline__ void a_hom_tile_dd(const RDesc& d, int64_t tile, CoefSrc cs,
+__device__ __forceinline__ void a_hom_tile_dd(const RDesc& d, int64_t tile, int cells, CoefSrc cs,
                                               const double2* __restrict__ u, ddouble* red,
                                               double* out) {
     const double h = d.h;
@@ -239,8 +332,8 @@ __device__ __forceinline__ void a_hom_tile_dd(const RDesc& d, int64_t tile, Coef
     ddouble acc[AHOM_NP];
 #pragma unroll
     for (int k = 0; k < AHOM_NP; ++k) acc[k] = ddouble{0.0, 0.0};
-    const int64_t base = tile * AHOM_TILE;
-    for (int t = threadIdx.x; t < AHOM_TILE; t += blockDim.x) {
+    const int64_t base = tile * cells;
+    for (int t = threadIdx.x; t < cells; t += blockDim.x) {
         const int64_t cidx = base + t;
         const int i = (int)(cidx >> d.log2n), j = (int)(cidx & (n - 1));
         double a;
@@ -321,43 +414,37 @@ __device__ __forceinline__ void a_hom_tile_dd(const RDesc& d, int64_t tile, Coef
     __syncthreads();
 }
 
-// Energy and flux forms from the double-double tile partials (16 doubles
-// per tile), by one whole warp; lane 0 writes A (rounded to FP64), A_lo (the
-// low parts, nullable) and Af (nullable).
+// Energy and flux forms from the double-double tile partials (16 doubles per
+// tile), by one block of eight warps, a warp per sum; writes A (rounded to
+// FP64), A_lo (the low parts, nullable) and Af (nullable: then only the energy
+// sums exist).  As one warp for all sums 1024 tiles took 211 us.
 template <int SCHEME>
 __device__ __forceinline__ void a_hom_finish_dd(const RDesc& d, const double* part, int nt,
-                                                double* A, double* Alo, double* Af) {
-    const int lane = threadIdx.x & 31;
-    ddouble s[AHOM_NP];
-#pragma unroll
-    for (int k = 0; k < AHOM_NP; ++k) {
+                                                ddouble* red, double* A, double* Alo, double* Af) {
+    const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+    if (Af || (k >= 1 && k <= 3)) {
         ddouble v{0.0, 0.0};
         for (int t = lane; t < nt; t += 32)
             v = dd_add(v, ddouble{part[(int64_t)t * 2 * AHOM_NP + 2 * k],
                                   part[(int64_t)t * 2 * AHOM_NP + 2 * k + 1]});
-        s[k] = dd_warp_sum(v);
+        v = dd_warp_sum(v);
+        if (lane == 0) red[k] = v;
     }
-    if (lane != 0) return;
+    __syncthreads();
+    if (threadIdx.x >= 8) return;
     // K L^2 is an integer below 2^53: exact
     const double kvol = (SCHEME == 0 ? 6.0 : 2.0) * (double)d.L * (double)d.L;
-    const ddouble e11 = dd_div(s[1], kvol), e12 = dd_div(s[2], kvol), e22 = dd_div(s[3], kvol);
-    A[0] = e11.hi;
-    A[1] = e12.hi;
-    A[2] = e12.hi;
-    A[3] = e22.hi;
-    if (Alo) {
-        Alo[0] = e11.lo;
-        Alo[1] = e12.lo;
-        Alo[2] = e12.lo;
-        Alo[3] = e22.lo;
-    }
-    if (Af) {
+    const int q = threadIdx.x;   // lanes 0 .. 3: entries of A, 4 .. 7: of Af
+    if (q < 4) {
+        const ddouble e = dd_div(red[q == 0 ? 1 : q == 3 ? 3 : 2], kvol);
+        A[q] = e.hi;
+        if (Alo) Alo[q] = e.lo;
+    } else if (Af) {
         const double nn = (double)d.n * (double)d.n;   // a power of two
-        const ddouble mean_a = dd_scale2(s[0], 1.0 / nn);
-        Af[0] = dd_add(mean_a, dd_div(s[4], kvol)).hi;   // P_11
-        Af[1] = dd_div(s[6], kvol).hi;                   // a_12: P_21
-        Af[2] = dd_div(s[5], kvol).hi;                   // a_21: P_12
-        Af[3] = dd_add(mean_a, dd_div(s[7], kvol)).hi;   // P_22
+        const ddouble mean_a = dd_scale2(red[0], 1.0 / nn);
+        // P_11, a_12: P_21, a_21: P_12, P_22
+        const ddouble f = dd_div(red[q == 4 ? 4 : q == 5 ? 6 : q == 6 ? 5 : 7], kvol);
+        Af[q - 4] = (q == 4 || q == 7) ? dd_add(mean_a, f).hi : f.hi;
     }
 }
 

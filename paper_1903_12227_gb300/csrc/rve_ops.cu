@@ -478,27 +478,33 @@ __global__ void __launch_bounds__(256, 3)
                         part + (int64_t)blockIdx.x * AHOM_NP);
 }
 
-// FP64 solves: double-double partials (16 doubles per tile).
-template <int SCHEME>
+// FP64 solves: double-double partials (16 doubles per tile), of the energy
+// form alone or of both forms.
+template <int SCHEME, bool FLUX>
 __global__ void __launch_bounds__(256) k_a_hom_part_dd(const RDesc* __restrict__ desc,
                                                        const int32_t* __restrict__ start, int batch,
-                                                       CoefSrc cs, const double2* __restrict__ u,
+                                                       int cells, CoefSrc cs,
+                                                       const double2* __restrict__ u,
                                                        double* __restrict__ part) {
-    __shared__ ddouble red[32 * AHOM_NP];
+    __shared__ ddouble red[FLUX ? 32 * AHOM_NP : 32];
     const int b = find_real(start, batch, blockIdx.x);
     const RDesc d = desc[b];
-    a_hom_tile_dd<SCHEME>(d, blockIdx.x - start[b], cs, u, red,
-                          part + (int64_t)blockIdx.x * 2 * AHOM_NP);
+    double* out = part + (int64_t)blockIdx.x * 2 * AHOM_NP;
+    if (FLUX) a_hom_tile_dd<SCHEME>(d, blockIdx.x - start[b], cells, cs, u, red, out);
+    else a_hom_tile_energy<SCHEME>(d, blockIdx.x - start[b], cells, cs, u, red, out);
 }
 
 template <int SCHEME>
-__global__ void k_a_hom_final_dd(const RDesc* __restrict__ desc, const int32_t* __restrict__ start,
-                                 int batch, const double* __restrict__ part, double* __restrict__ A,
-                                 double* __restrict__ Alo, double* __restrict__ Af) {
-    const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (b >= batch) return;
+__global__ void __launch_bounds__(256) k_a_hom_final_dd(const RDesc* __restrict__ desc,
+                                                        const int32_t* __restrict__ start,
+                                                        const double* __restrict__ part,
+                                                        double* __restrict__ A,
+                                                        double* __restrict__ Alo,
+                                                        double* __restrict__ Af) {
+    __shared__ ddouble red[AHOM_NP];
+    const int b = blockIdx.x;
     const RDesc d = desc[b];
-    a_hom_finish_dd<SCHEME>(d, part + (int64_t)start[b] * 2 * AHOM_NP, start[b + 1] - start[b],
+    a_hom_finish_dd<SCHEME>(d, part + (int64_t)start[b] * 2 * AHOM_NP, start[b + 1] - start[b], red,
                             A + 4 * (int64_t)b, Alo ? Alo + 4 * (int64_t)b : nullptr,
                             Af ? Af + 4 * (int64_t)b : nullptr);
 }
@@ -689,12 +695,14 @@ cudaError_t launch_a_hom(const Plan& p, void* ws, const uint32_t* mask, const do
     const bool lumped = scheme == RVE_Q1_LUMPED;
     const int gf = (p.batch + 7) / 8;
     if (precision == RVE_FP64) {
-        if (lumped) k_a_hom_part_dd<1><<<p.tilesA, 256, 0, s>>>(desc, start, p.batch, cs, uu, part);
-        else k_a_hom_part_dd<0><<<p.tilesA, 256, 0, s>>>(desc, start, p.batch, cs, uu, part);
+        const int threads = std::min(256, p.cellsA);
+        auto parts = lumped ? (A_flux ? k_a_hom_part_dd<1, true> : k_a_hom_part_dd<1, false>)
+                            : (A_flux ? k_a_hom_part_dd<0, true> : k_a_hom_part_dd<0, false>);
+        parts<<<p.tilesA, threads, 0, s>>>(desc, start, p.batch, p.cellsA, cs, uu, part);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        if (lumped) k_a_hom_final_dd<1><<<gf, 256, 0, s>>>(desc, start, p.batch, part, A, A_lo, A_flux);
-        else k_a_hom_final_dd<0><<<gf, 256, 0, s>>>(desc, start, p.batch, part, A, A_lo, A_flux);
+        if (lumped) k_a_hom_final_dd<1><<<p.batch, 256, 0, s>>>(desc, start, part, A, A_lo, A_flux);
+        else k_a_hom_final_dd<0><<<p.batch, 256, 0, s>>>(desc, start, part, A, A_lo, A_flux);
     } else {
         const int32_t* start2 = reinterpret_cast<const int32_t*>(w + p.o_startA2);
         if (lumped) k_a_hom_strip<1><<<p.tilesA2, 256, 0, s>>>(desc, start2, p.batch, cs, uu, part);
