@@ -675,17 +675,23 @@ __global__ void __launch_bounds__(T3) k3_rhs(Grp g, Cells3T<double> cs, double2*
 // buffer per line; AXIS 1: y lines (stride n), the G lines of a block side
 // by side so that each load instruction reads consecutive nodes, and their
 // buffers interleaved element by element so that the lanes of a warp (G
-// consecutive lines at the same element) touch consecutive words.  With
-// `rd` set, also the block's partials of rd.dst per component (the r.z of
-// CG).
-template <int LOG2N, int AXIS, typename V>
+// consecutive lines at the same element) touch consecutive words.
+//
+// STEP: the last x pass of a CG step, which forms the new direction from the
+// preconditioned residual without storing it: with p the old direction, e +=
+// alpha p and p = scale H src + beta p (e and p are the step's, src is left).
+// r.z, and so beta, comes from the z solve one pass earlier.  Before, the pass
+// stored z and read r for r.z, a launch formed p = z + beta p, and e += alpha p
+// read p beside the residual's update: 177 bytes per node and step in FP32,
+// 145 now; 15 realizations of 64^3 37.4 -> 33.2 ms.
+template <typename T> __device__ __forceinline__ T alpha_of(const MixScal& s, int k);
+template <typename T> __device__ __forceinline__ T beta_of(const MixScal& s, int k);
+template <int LOG2N, int AXIS, bool STEP, typename V>
 __global__ void __launch_bounds__(256) k3_lines(Grp g, Tables tb, const V* src, V* dst,
-                                                typename ScalarOf<V>::T scale,
-                                                const V* __restrict__ rd, double* part,
+                                                typename ScalarOf<V>::T scale, V* __restrict__ e,
                                                 const MixScal* sc) {
     typedef typename ScalarOf<V>::T T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ double red[16];
     int lb;
     const int u = unit_of(g, lb);
     const U3 d = g.desc[u];   // issued before the flag test
@@ -704,31 +710,43 @@ __global__ void __launch_bounds__(256) k3_lines(Grp g, Tables tb, const V* src, 
 #pragma unroll
     for (int mm = 0; mm < 8; ++mm) w[mm] = src[base + (t + mm * TL) * stride];
     fft_reg<FFT_TO_BOTH, LOG2N, BS>(w, buf, LOG2N, t, twiddles<V>(tb, n), true);
-    T ax = 0, ay = 0;
-#pragma unroll
-    for (int mm = 0; mm < 8; ++mm) {
-        const int kx = t + mm * TL;
-        const V hv = hartley_pair(w[mm], buf[pidx((n - kx) & (n - 1)) * BS]);
-        const V o = mk<V>(scale * hv.x, scale * hv.y);
-        dst[base + (int64_t)kx * stride] = o;
-        if (rd) {
-            const V r = rd[base + (int64_t)kx * stride];
-            ax = fma(r.x, o.x, ax);
-            ay = fma(r.y, o.y, ay);
-        }
+    T ax = 0, ay = 0, bx = 0, by = 0;
+    if (STEP) {
+        ax = alpha_of<T>(sc[u], 0);
+        ay = alpha_of<T>(sc[u], 1);
+        bx = beta_of<T>(sc[u], 0);
+        by = beta_of<T>(sc[u], 1);
     }
-    if (rd) {   // block-uniform
-        double sx = 0.0, sy = 0.0;
-        block_pair_sum(ax, ay, red, sx, sy);
-        if (threadIdx.x == 0) {
-            part[d.part_off + 2 * lb] = sx;
-            part[d.part_off + 2 * lb + 1] = sy;
+    // in halves of four: a half's loads before its stores
+#pragma unroll
+    for (int h = 0; h < 8; h += 4) {
+        V po[4], eo[4];
+        if (STEP) {
+#pragma unroll
+            for (int mm = 0; mm < 4; ++mm) {
+                const int64_t node = base + (int64_t)(t + (h + mm) * TL) * stride;
+                po[mm] = dst[node];
+                eo[mm] = e[node];
+            }
+        }
+#pragma unroll
+        for (int mm = 0; mm < 4; ++mm) {
+            const int kx = t + (h + mm) * TL;
+            const int64_t node = base + (int64_t)kx * stride;
+            const V hv = hartley_pair(w[h + mm], buf[pidx((n - kx) & (n - 1)) * BS]);
+            V o = mk<V>(scale * hv.x, scale * hv.y);
+            if (STEP) {
+                e[node] = mk<V>(fma(ax, po[mm].x, eo[mm].x), fma(ay, po[mm].y, eo[mm].y));
+                o = mk<V>(fma(bx, po[mm].x, o.x), fma(by, po[mm].y, o.y));
+            }
+            dst[node] = o;
         }
     }
 }
 
 // Tridiagonal solves along z after the x and y transforms; writes M^{-1} t
-// / n in place.  The n^2 columns (kx, ky) of a unit are numbered kc = ky n +
+// / n in place and, with `part`, the partials of r.z (the transforms being
+// orthogonal up to n, r.z is a sum over the transformed residual).  The n^2 columns (kx, ky) of a unit are numbered kc = ky n +
 // kx, so column kc, row r sits at r n^2 + kc; a block takes ZC consecutive
 // columns (ZSEG rows per thread, ZC x n / ZSEG = 512 threads).  The filter
 // root of (kx, ky) solves rho + 1/rho = 2 + lambda(kx) + lambda(ky) + delta
@@ -741,11 +759,13 @@ template <typename T> __device__ __forceinline__ T filter_root_t(T mu) {
 }
 template <int LOG2N, typename V>
 __global__ void __launch_bounds__(Z_THREADS) k3_zsolve(Grp g, Tables tb, double delta,
-                                                       V* __restrict__ v, const MixScal* sc) {
+                                                       V* __restrict__ v, double* part,
+                                                       const MixScal* sc) {
     typedef typename ScalarOf<V>::T T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[64];
     __shared__ T csc[1];
+    double pz[2] = {0.0, 0.0};   // thread 0: the block's share of t.(M^-1 t / n)
     int lb;
     const int u = unit_of(g, lb);
     const U3 d = g.desc[u];   // issued before the flag test
@@ -766,7 +786,11 @@ __global__ void __launch_bounds__(Z_THREADS) k3_zsolve(Grp g, Tables tb, double 
             return (ky == 0 && delta == 0.0) ? rho_table<T>(tb, n)[kx]
                                              : filter_root_t<T>(lapT[kx] + lapT[ky] + dc);
         },
-        cd, c0, reinterpret_cast<V*>(smem_raw), tb, delta, red, nullptr, csc);
+        cd, c0, reinterpret_cast<V*>(smem_raw), tb, delta, red, part ? pz : nullptr, csc);
+    if (part && threadIdx.x == 0) {   // r.z = t.(M^-1 t / n) / n, t = Hy Hx r
+        part[d.part_off + 2 * lb] = pz[0] / (double)n;
+        part[d.part_off + 2 * lb + 1] = pz[1] / (double)n;
+    }
 }
 
 // ------------------------------------------------------------- A_hom --
@@ -1019,10 +1043,8 @@ __global__ void __launch_bounds__(256) k3_scalar(int first, const U3* __restrict
 }
 
 // The step scalars in the cycle's precision.
-template <typename T> __device__ __forceinline__ T alpha_of(const MixScal& s, int k);
 template <> __device__ __forceinline__ double alpha_of<double>(const MixScal& s, int k) { return s.alpha[k]; }
 template <> __device__ __forceinline__ float alpha_of<float>(const MixScal& s, int k) { return s.alpha_f[k]; }
-template <typename T> __device__ __forceinline__ T beta_of(const MixScal& s, int k);
 template <> __device__ __forceinline__ double beta_of<double>(const MixScal& s, int k) { return s.beta[k]; }
 template <> __device__ __forceinline__ float beta_of<float>(const MixScal& s, int k) { return s.beta_f[k]; }
 
@@ -1052,11 +1074,11 @@ __global__ void __launch_bounds__(T3) k3_start(Grp g, const MixScal* scs,
     p[node] = mk<V>((T)0, (T)0);
 }
 
-// e += alpha p; r -= alpha q; partials |r|^2.  Four nodes per thread.
+// r -= alpha q; partials |r|^2.  Four nodes per thread.  (e += alpha p follows
+// in the step's last line pass, which reads p anyway.)
 template <typename V>
-__global__ void __launch_bounds__(T3) k3_axpy(Grp g, const MixScal* scs, V* __restrict__ e,
-                                              V* __restrict__ r, const V* __restrict__ p,
-                                              const V* __restrict__ q, double* part) {
+__global__ void __launch_bounds__(T3) k3_update(Grp g, const MixScal* scs, V* __restrict__ r,
+                                                const V* __restrict__ q, double* part) {
     typedef typename ScalarOf<V>::T T;
     __shared__ double red[16];
     int lb;
@@ -1066,19 +1088,21 @@ __global__ void __launch_bounds__(T3) k3_axpy(Grp g, const MixScal* scs, V* __re
     if (sc.done) return;
     const T ax_ = alpha_of<T>(sc, 0), ay_ = alpha_of<T>(sc, 1);
     T sx = 0, sy = 0;
+    V qq[4], rr[4];
 #pragma unroll
     for (int mm = 0; mm < 4; ++mm) {
         const int64_t node = d.off + (int64_t)lb * (4 * T3) + mm * T3 + threadIdx.x;
-        const V pp = p[node], qq = q[node];
-        V ee = e[node], rr = r[node];
-        ee.x = fma(ax_, pp.x, ee.x);
-        ee.y = fma(ay_, pp.y, ee.y);
-        rr.x = fma(-ax_, qq.x, rr.x);
-        rr.y = fma(-ay_, qq.y, rr.y);
-        e[node] = ee;
-        r[node] = rr;
-        sx = fma(rr.x, rr.x, sx);
-        sy = fma(rr.y, rr.y, sy);
+        qq[mm] = q[node];
+        rr[mm] = r[node];
+    }
+#pragma unroll
+    for (int mm = 0; mm < 4; ++mm) {
+        const int64_t node = d.off + (int64_t)lb * (4 * T3) + mm * T3 + threadIdx.x;
+        rr[mm].x = fma(-ax_, qq[mm].x, rr[mm].x);
+        rr[mm].y = fma(-ay_, qq[mm].y, rr[mm].y);
+        r[node] = rr[mm];
+        sx = fma(rr[mm].x, rr[mm].x, sx);
+        sy = fma(rr[mm].y, rr[mm].y, sy);
     }
     double tx = 0.0, ty = 0.0;
     block_pair_sum(sx, sy, red, tx, ty);
@@ -1088,29 +1112,13 @@ __global__ void __launch_bounds__(T3) k3_axpy(Grp g, const MixScal* scs, V* __re
     }
 }
 
-// p = z + beta p.  Four nodes per thread.
-template <typename V>
-__global__ void __launch_bounds__(T3) k3_xpby(Grp g, const MixScal* scs, const V* __restrict__ z,
-                                              V* __restrict__ p) {
-    typedef typename ScalarOf<V>::T T;
-    int lb;
-    const int u = unit_of(g, lb);
-    const U3 d = g.desc[u];   // issued before the flag test
-    const MixScal& sc = scs[u];
-    if (sc.done) return;
-    const T bx = beta_of<T>(sc, 0), by = beta_of<T>(sc, 1);
-#pragma unroll
-    for (int mm = 0; mm < 4; ++mm) {
-        const int64_t node = d.off + (int64_t)lb * (4 * T3) + mm * T3 + threadIdx.x;
-        const V zz = z[node], pp = p[node];
-        p[node] = mk<V>(fma(bx, pp.x, zz.x), fma(by, pp.y, zz.y));
-    }
-}
-
-// End of a cycle: u += s e (components that iterated).
+// End of a cycle: u += s (e + alpha p) (components that iterated; the last
+// step's alpha p is still due: a unit that is done skips the line pass, and
+// alpha is 0 for a component that ended before).
 template <typename V>
 __global__ void __launch_bounds__(T3) k3_accum(Grp g, const MixScal* scs, const V* __restrict__ e,
-                                               double2* __restrict__ uv) {
+                                               const V* __restrict__ p, double2* __restrict__ uv) {
+    typedef typename ScalarOf<V>::T T;
     int lb;
     const int u = unit_of(g, lb);
     const U3 d = g.desc[u];   // issued before the flag test
@@ -1118,7 +1126,10 @@ __global__ void __launch_bounds__(T3) k3_accum(Grp g, const MixScal* scs, const 
     if (sc.outer_done) return;
     const int64_t node = d.off + lb * T3 + threadIdx.x;
     const double sx = sc.cdone[0] ? 0.0 : sc.s[0], sy = sc.cdone[1] ? 0.0 : sc.s[1];
-    const V ee = e[node];
+    V ee = e[node];
+    const V pp = p[node];
+    ee.x = fma(alpha_of<T>(sc, 0), pp.x, ee.x);
+    ee.y = fma(alpha_of<T>(sc, 1), pp.y, ee.y);
     double2 w = uv[node];
     w.x = fma(sx, (double)ee.x, w.x);
     w.y = fma(sy, (double)ee.y, w.y);
@@ -1370,11 +1381,13 @@ static rve_status setup3(const Plan3& p, char* w, cudaStream_t s, bool tables) {
     return fill_tables(ws.tables(), p.max_log2n, s) == cudaSuccess ? RVE_OK : RVE_ECUDA;
 }
 
-// dst = B^{-1} src for the units of group g; src is read by the first pass
-// only (it may equal dst).  With `rd`, the units' partials of rd.dst.
+// The preconditioner's passes over the units of group g, z = M^-1 Hy Hx src / n
+// (half 1, with the partials of src.B^-1 src if `rz`), and dst from z (half 2):
+// B^-1 src without `e`, the step's new direction and iterate with it.  src is
+// read by the first pass only (it may equal z).
 template <int LG, typename V>
-static cudaError_t precond3_t(const Ws3& ws, const Group3& g, double delta, const V* src, V* dst,
-                              const V* rd, const MixScal* sc, cudaStream_t s) {
+static cudaError_t precond3_t(const Ws3& ws, const Group3& g, double delta, const V* src, V* z, V* dst,
+                              V* e, bool rz, int half, const MixScal* sc, cudaStream_t s) {
     typedef typename ScalarOf<V>::T T;
     constexpr int n = 1 << LG, TL = n / 8;
     const int G = 256 / TL;
@@ -1382,47 +1395,54 @@ static cudaError_t precond3_t(const Ws3& ws, const Group3& g, double delta, cons
     const int lines = (n * n) / G;
     constexpr int ZC = zcols<LG>(), ZP = n / ZSEG;
     const size_t zsmem = (size_t)(2 * ZC + 2) * ZP * sizeof(V);
-    cudaError_t e = cudaFuncSetAttribute(k3_lines<LG, 2, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k3_lines<LG, 1, V>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    auto lx = k3_lines<LG, 2, false, V>;
+    auto ly = k3_lines<LG, 1, false, V>;
+    auto ls = k3_lines<LG, 2, true, V>;
+    cudaError_t er = cudaSuccess;
+    for (auto k : {lx, ly, ls})
+        if (er == cudaSuccess) er = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (er != cudaSuccess) return er;
     const Tables tb = ws.tables();
-    double* part = ws.part();
     const Grp gl = ws.grp(g, lines);
     const unsigned bl = nblocks(g, lines);
-    {
-        Span3 sp(s, P3_LINES);
-        k3_lines<LG, 2, V><<<bl, 256, smem, s>>>(gl, tb, src, dst, (T)1, nullptr, nullptr, sc);
+    if (half & 1) {
+        {
+            Span3 sp(s, P3_LINES);
+            lx<<<bl, 256, smem, s>>>(gl, tb, src, z, (T)1, nullptr, sc);
+        }
+        {
+            Span3 sp(s, P3_LINES);
+            ly<<<bl, 256, smem, s>>>(gl, tb, z, z, (T)1, nullptr, sc);
+        }
+        {
+            Span3 sp(s, P3_ZSOLVE);
+            k3_zsolve<LG, V><<<nblocks(g, n * n / ZC), Z_THREADS, zsmem, s>>>(
+                ws.grp(g, n * n / ZC), tb, delta, z, rz ? ws.part() : nullptr, sc);
+        }
+        note_launch(3);
     }
-    {
-        Span3 sp(s, P3_LINES);
-        k3_lines<LG, 1, V><<<bl, 256, smem, s>>>(gl, tb, dst, dst, (T)1, nullptr, nullptr, sc);
+    if (half & 2) {
+        {
+            Span3 sp(s, P3_LINES);
+            ly<<<bl, 256, smem, s>>>(gl, tb, z, z, (T)1, nullptr, sc);
+        }
+        {
+            Span3 sp(s, P3_LINES);
+            (e ? ls : lx)<<<bl, 256, smem, s>>>(gl, tb, z, dst, (T)(1.0 / (double)n), e, sc);
+        }
+        note_launch(2);
     }
-    {
-        Span3 sp(s, P3_ZSOLVE);
-        k3_zsolve<LG, V><<<nblocks(g, n * n / ZC), Z_THREADS, zsmem, s>>>(
-            ws.grp(g, n * n / ZC), tb, delta, dst, sc);
-    }
-    {
-        Span3 sp(s, P3_LINES);
-        k3_lines<LG, 1, V><<<bl, 256, smem, s>>>(gl, tb, dst, dst, (T)1, nullptr, nullptr, sc);
-    }
-    {
-        Span3 sp(s, P3_LINES);
-        k3_lines<LG, 2, V><<<bl, 256, smem, s>>>(gl, tb, dst, dst, (T)(1.0 / (double)n), rd, part, sc);
-    }
-    note_launch(5);
     return cudaGetLastError();
 }
 
 template <typename V>
-static cudaError_t precond3(const Ws3& ws, const Group3& g, double delta, const V* src, V* dst,
-                            cudaStream_t s, const V* rd = nullptr, const MixScal* sc = nullptr) {
+static cudaError_t precond3(const Ws3& ws, const Group3& g, double delta, const V* src, V* z, V* dst,
+                            V* e, bool rz, int half, const MixScal* sc, cudaStream_t s) {
     switch (g.log2n) {
-        case 5: return precond3_t<5, V>(ws, g, delta, src, dst, rd, sc, s);
-        case 6: return precond3_t<6, V>(ws, g, delta, src, dst, rd, sc, s);
-        case 7: return precond3_t<7, V>(ws, g, delta, src, dst, rd, sc, s);
-        default: return precond3_t<8, V>(ws, g, delta, src, dst, rd, sc, s);
+        case 5: return precond3_t<5, V>(ws, g, delta, src, z, dst, e, rz, half, sc, s);
+        case 6: return precond3_t<6, V>(ws, g, delta, src, z, dst, e, rz, half, sc, s);
+        case 7: return precond3_t<7, V>(ws, g, delta, src, z, dst, e, rz, half, sc, s);
+        default: return precond3_t<8, V>(ws, g, delta, src, z, dst, e, rz, half, sc, s);
     }
 }
 
@@ -1484,15 +1504,22 @@ static rve_status solve_units(const Plan3& p, char* w, Cells3T<double> cs64,
         Span3 sp(s, P3_VECTOR);
         launch();
     };
-    // partial pairs per unit: n^3 >> shift (rhs: 256 nodes per block; axpy:
-    // 1024; stiffness and the last line pass: 2048)
-    constexpr int SH_RHS = 8, SH_STIFF = 11, SH_AXPY = 10, SH_LINES = 11;
-    static_assert(2 * T3 * SZ == (1 << SH_STIFF) && 4 * T3 == (1 << SH_AXPY) && T3 == (1 << SH_RHS),
+    // partial pairs per unit: n^3 >> shift (rhs: 256 nodes per block; update:
+    // 1024; stiffness: 2048; z solve: 8192)
+    constexpr int SH_RHS = 8, SH_STIFF = 11, SH_AXPY = 10, SH_Z = 13;
+    static_assert(2 * T3 * SZ == (1 << SH_STIFF) && 4 * T3 == (1 << SH_AXPY) && T3 == (1 << SH_RHS) &&
+                      Z_THREADS * ZSEG == (1 << SH_Z),
                   "partial counts");
     auto scalar = [&](const Group3& g, int what, int shift) {
         Span3 sp(s, P3_SCALAR);
         k3_scalar<<<g.count, 256, 0, s>>>(g.first, ws.desc(), sc, part, what, shift, sa);
         note_launch();
+    };
+    // z = B^-1 r with r.z, then the scalar step, then e += alpha p, p = z + beta p
+    auto direction = [&](const Group3& g, int what) -> bool {
+        if (precond3<V>(ws, g, o.delta, r, z, pp, e, true, 1, sc, s) != cudaSuccess) return false;
+        scalar(g, what, SH_Z);
+        return precond3<V>(ws, g, o.delta, r, z, pp, e, true, 2, sc, s) == cudaSuccess;
     };
     auto per_group = [&](auto&& fn) -> rve_status {
         for (const Group3& g : p.groups) {
@@ -1552,12 +1579,8 @@ static rve_status solve_units(const Plan3& p, char* w, Cells3T<double> cs64,
         st = per_group([&](const Group3& g) {
             const int per = (int)(nodes_of(g) / T3);
             vec_step([&] { k3_start<V><<<nblocks(g, per), T3, 0, s>>>(ws.grp(g, per), sc, r64, r, e, pp); });
-            if (precond3<V>(ws, g, o.delta, r, z, s, r, sc) != cudaSuccess) return RVE_ECUDA;
-            scalar(g, M_RHO0, SH_LINES);
-            const int per4 = per / 4;
-            vec_step([&] { k3_xpby<V><<<nblocks(g, per4), T3, 0, s>>>(ws.grp(g, per4), sc, z, pp); });
-            note_launch(2);
-            return RVE_OK;
+            note_launch();
+            return direction(g, M_RHO0) ? RVE_OK : RVE_ECUDA;   // alpha = beta = 0, e = p = 0
         });
         if (st != RVE_OK) return st;
         for (int it = 1;; ++it) {
@@ -1568,14 +1591,11 @@ static rve_status solve_units(const Plan3& p, char* w, Cells3T<double> cs64,
                     return RVE_ECUDA;
                 scalar(g, M_ALPHA, SH_STIFF);
                 vec_step([&] {
-                    k3_axpy<V><<<nblocks(g, per4), T3, 0, s>>>(ws.grp(g, per4), sc, e, r, pp, q, part);
+                    k3_update<V><<<nblocks(g, per4), T3, 0, s>>>(ws.grp(g, per4), sc, r, q, part);
                 });
                 scalar(g, M_CONV, SH_AXPY);
-                if (precond3<V>(ws, g, o.delta, r, z, s, r, sc) != cudaSuccess) return RVE_ECUDA;
-                scalar(g, M_BETA, SH_LINES);
-                vec_step([&] { k3_xpby<V><<<nblocks(g, per4), T3, 0, s>>>(ws.grp(g, per4), sc, z, pp); });
-                note_launch(2);
-                return RVE_OK;
+                note_launch();
+                return direction(g, M_BETA) ? RVE_OK : RVE_ECUDA;
             });
             if (st != RVE_OK) return st;
             if (it % every == 0) {
@@ -1586,7 +1606,7 @@ static rve_status solve_units(const Plan3& p, char* w, Cells3T<double> cs64,
         }
         st = per_group([&](const Group3& g) {
             const int per = (int)(nodes_of(g) / T3);
-            vec_step([&] { k3_accum<V><<<nblocks(g, per), T3, 0, s>>>(ws.grp(g, per), sc, e, uv); });
+            vec_step([&] { k3_accum<V><<<nblocks(g, per), T3, 0, s>>>(ws.grp(g, per), sc, e, pp, uv); });
             note_launch();
             return RVE_OK;
         });
@@ -1707,7 +1727,7 @@ rve_status rve3_apply_precond(const rve_realization* r, int32_t batch, double de
         note_launch();
     }
     for (const Group3& g : p.groups)
-        if (precond3<double2>(W, g, delta, v, v, s) != cudaSuccess) return RVE_ECUDA;
+        if (precond3<double2>(W, g, delta, v, v, v, nullptr, false, 3, nullptr, s) != cudaSuccess) return RVE_ECUDA;
     for (const Group3& g : p.groups) {
         const int per = (int)(nodes_of(g) / T3);
         k3_join<<<nblocks(g, per), T3, 0, s>>>(W.grp(g, per), v, y);
