@@ -50,20 +50,6 @@
 
 namespace rve {
 
-// ------------------------------------------------------------ element --
-// Entry (a, b) of the element matrix (local corners 4 a1 + 2 a2 + a3).
-template <int SCHEME>
-__host__ __device__ __forceinline__ double e3(int a, int b, double h) {
-    auto m1 = [&](int x, int y) {
-        return SCHEME == 0 ? h * (x == y ? 1.0 / 3.0 : 1.0 / 6.0) : (x == y ? 0.5 * h : 0.0);
-    };
-    auto k1 = [&](int x, int y) { return (x == y ? 1.0 : -1.0) / h; };
-    const int a1 = a >> 2, a2 = (a >> 1) & 1, a3 = a & 1;
-    const int b1 = b >> 2, b2 = (b >> 1) & 1, b3 = b & 1;
-    return k1(a1, b1) * m1(a2, b2) * m1(a3, b3) + m1(a1, b1) * k1(a2, b2) * m1(a3, b3) +
-           m1(a1, b1) * m1(a2, b2) * k1(a3, b3);
-}
-
 // Descriptor of one unit (a corrector pair of a realization).
 struct U3 {
     int32_t n, log2n, pair, pad2;
@@ -642,18 +628,13 @@ __global__ void __launch_bounds__(T3) k3_rhs(Grp g, Cells3T<double> cs, double2*
         a[c] = cs.coef ? cs.coef[d.cell_off + idx] : two_values<double>(d, cs.mask[d.cell_off + idx] != 0);
     }
     const double q = 0.25 * d.h * d.h;
-    double v[3];
-#pragma unroll
-    for (int ax = 0; ax < 3; ++ax) {
-        double lo = 0.0, hi = 0.0;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            if ((c >> (2 - ax)) & 1) hi += a[c];
-            else lo += a[c];
-        }
-        v[ax] = q * (lo - hi);
+    double2 out;
+    if (d.pair == 0) {   // cells summed along the third axis, then differences along the first two
+        const double t00 = a[0] + a[1], t01 = a[2] + a[3], t10 = a[4] + a[5], t11 = a[6] + a[7];
+        out = make_double2(q * ((t00 + t01) - (t10 + t11)), q * ((t00 + t10) - (t01 + t11)));
+    } else {
+        out = make_double2(q * (((a[0] + a[2]) + (a[4] + a[6])) - ((a[1] + a[3]) + (a[5] + a[7]))), 0.0);
     }
-    const double2 out = d.pair == 0 ? make_double2(v[0], v[1]) : make_double2(v[2], 0.0);
     f[d.off + local] = out;
     if (part) {
         DotAcc<double> dx, dy;
@@ -683,7 +664,7 @@ __global__ void __launch_bounds__(T3) k3_rhs(Grp g, Cells3T<double> cs, double2*
 // r.z, and so beta, comes from the z solve one pass earlier.  Before, the pass
 // stored z and read r for r.z, a launch formed p = z + beta p, and e += alpha p
 // read p beside the residual's update: 177 bytes per node and step in FP32,
-// 145 now; 15 realizations of 64^3 37.4 -> 33.2 ms.
+// 145 now; 15 realizations of 64^3 37.4 -> 33.4 ms.
 template <typename T> __device__ __forceinline__ T alpha_of(const MixScal& s, int k);
 template <typename T> __device__ __forceinline__ T beta_of(const MixScal& s, int k);
 template <int LOG2N, int AXIS, bool STEP, typename V>
@@ -794,94 +775,137 @@ __global__ void __launch_bounds__(Z_THREADS) k3_zsolve(Grp g, Tables tb, double 
 }
 
 // ------------------------------------------------------------- A_hom --
-// Per tile of T3 cells, partial sums of sum a_c, the energy terms
+// Per tile of 4 T3 cells, partial sums of sum a_c, the energy terms
 // a_c v_i^T E v_j (ij = 11 12 13 22 23 33) and the flux terms a_c int_c
 // d_j (x_i + phi_i) (ij = 11 12 13 21 22 23 31 32 33), v_i = xi_i + P_c u_i.
+// The element matrix is diagonal in the sum / difference basis of each axis
+// (K1 has 0 and 2/h, M1 has h/2 and h/6, lumped h/2), so with w the 8 signed
+// sums of a cell's corner values
+//     v^T E v' = (1/8) sum_b lambda_|b| w_b w'_b,   lambda = 0, h/2, h/3, h/6
+// (lumped 0, h/2, h, 3h/2), and int_c d_j v = (h^2/4) w_{e_j}.  A thread walks
+// up four planes, so that a plane's sums serve two cells: 128 FP64 operations
+// per cell instead of 700 with the 8 x 8 products; 15 x 64^3 cells 3.2 -> 1.0 ms.
 // Launched over realizations (the pair-0 unit descriptors); u is the ABI
 // layout [nodes][3].
-constexpr int A3_NP = 16;
+constexpr int A3_NP = 16, A3_PLANES = 4;
 template <int SCHEME>
 __global__ void __launch_bounds__(T3) k3_a_hom_part(Grp g, Cells3T<double> cs,
                                                     const double* __restrict__ u3,
                                                     double* __restrict__ part) {
-    __shared__ double red[8];
+    __shared__ double red[T3 / 32][A3_NP];
     int lb;
     const int un = unit_of(g, lb);
     const U3& d = g.desc[un];
-    const int cell = lb * T3 + threadIdx.x;
-    const int n = d.n;
-    const int i = cell >> (2 * d.log2n), j = (cell >> d.log2n) & (n - 1), k = cell & (n - 1);
+    const int lg = d.log2n, n = d.n;
+    const int first = lb * T3;   // (plane group, j, k)
+    const int i0 = (first >> (2 * lg)) * A3_PLANES;
+    const int jk = (first & ((1 << (2 * lg)) - 1)) + threadIdx.x;
+    const int j = jk >> lg, k = jk & (n - 1);
     const double h = d.h;
-    const double a = cs.coef ? cs.coef[d.cell_off + cell] : two_values<double>(d, cs.mask[d.cell_off + cell] != 0);
-    double v[3][8];
+    const double* __restrict__ uu = u3 + 3 * d.cell_off;
+    // sum, k-, j- and jk-difference of a plane's four corners, per corrector
+    auto plane = [&](int i, double (&P)[3][4]) {
+        const int64_t a = 3 * (int64_t)l3(d, i, j, k), b = 3 * (int64_t)l3(d, i, j, k + 1);
+        const int64_t c = 3 * (int64_t)l3(d, i, j + 1, k), e = 3 * (int64_t)l3(d, i, j + 1, k + 1);
 #pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const int64_t gi = 3 * (d.cell_off + l3(d, i + (b >> 2), j + ((b >> 1) & 1), k + (b & 1)));
-        v[0][b] = u3[gi] + h * (double)(b >> 2);
-        v[1][b] = u3[gi + 1] + h * (double)((b >> 1) & 1);
-        v[2][b] = u3[gi + 2] + h * (double)(b & 1);
-    }
-    double Ev[3][8];
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-            double s = 0.0;
-#pragma unroll
-            for (int b = 0; b < 8; ++b) s = fma(e3<SCHEME>(r, b, h), v[c][b], s);
-            Ev[c][r] = s;
+        for (int x = 0; x < 3; ++x) {
+            const double u00 = uu[a + x], u01 = uu[b + x], u10 = uu[c + x], u11 = uu[e + x];
+            const double p0 = u00 + u01, p1 = u10 + u11, q0 = u01 - u00, q1 = u11 - u10;
+            P[x][0] = p0 + p1;
+            P[x][1] = q0 + q1;
+            P[x][2] = p1 - p0;
+            P[x][3] = q1 - q0;
         }
+    };
+    const double l1 = h / 16.0, l2 = SCHEME == 0 ? h / 24.0 : h / 8.0, l3_ = SCHEME == 0 ? h / 48.0 : 3.0 * h / 16.0;
     double val[A3_NP];
-    val[0] = a;
-    int q = 1;
 #pragma unroll
-    for (int x = 0; x < 3; ++x)
+    for (int q = 0; q < A3_NP; ++q) val[q] = 0.0;
+    double P[3][4];
+    plane(i0, P);
+#pragma unroll 1
+    for (int i = i0; i < i0 + A3_PLANES; ++i) {
+        const int cell = l3(d, i, j, k);
+        const double a = cs.coef ? cs.coef[d.cell_off + cell] : two_values<double>(d, cs.mask[d.cell_off + cell] != 0);
+        double N[3][4], w[3][7];   // w: k, j, i, jk, ik, ij, ijk
+        plane(i + 1, N);
 #pragma unroll
-        for (int y = x; y < 3; ++y) {
-            double s = 0.0;
+        for (int x = 0; x < 3; ++x) {
+            w[x][0] = P[x][1] + N[x][1];
+            w[x][1] = P[x][2] + N[x][2];
+            w[x][2] = N[x][0] - P[x][0];
+            w[x][3] = P[x][3] + N[x][3];
+            w[x][4] = N[x][1] - P[x][1];
+            w[x][5] = N[x][2] - P[x][2];
+            w[x][6] = N[x][3] - P[x][3];
+            w[x][2 - x] += 4.0 * h;   // xi_x
 #pragma unroll
-            for (int r = 0; r < 8; ++r) s = fma(v[x][r], Ev[y][r], s);
-            val[q++] = a * s;
+            for (int q = 0; q < 4; ++q) P[x][q] = N[x][q];
+        }
+        const double a1 = a * l1, a2 = a * l2, a3 = a * l3_;
+        val[0] += a;
+        int q = 1;
+#pragma unroll
+        for (int x = 0; x < 3; ++x) {
+            double s[7];
+#pragma unroll
+            for (int b = 0; b < 7; ++b) s[b] = (b < 3 ? a1 : b < 6 ? a2 : a3) * w[x][b];
+#pragma unroll
+            for (int y = x; y < 3; ++y) {
+#pragma unroll
+                for (int b = 0; b < 7; ++b) val[q] = fma(s[b], w[y][b], val[q]);
+                ++q;
+            }
         }
 #pragma unroll
-    for (int x = 0; x < 3; ++x)
+        for (int x = 0; x < 3; ++x)
 #pragma unroll
-        for (int y = 0; y < 3; ++y) {
-            double s = 0.0;
+            for (int y = 0; y < 3; ++y) {
+                val[q] = fma(a, w[x][2 - y], val[q]);
+                ++q;
+            }
+    }
 #pragma unroll
-            for (int b = 0; b < 8; ++b) s += ((b >> (2 - y)) & 1) ? v[x][b] : -v[x][b];
-            val[q++] = a * 0.25 * h * h * s;
+    for (int q = 7; q < A3_NP; ++q) val[q] *= 0.25 * h * h;
+    // the 16 sums over the warp in 16 additions per lane: at each step half of
+    // the lanes keep half of the sums; lane l ends with sum bit-reverse(l / 2)
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+    for (int w = 8, o = 16; w >= 1; w >>= 1, o >>= 1) {
+        const bool hi = lane & o;
+#pragma unroll
+        for (int q = 0; q < w; ++q) {
+            const double send = hi ? val[q] : val[q + w], keep = hi ? val[q + w] : val[q];
+            val[q] = keep + __shfl_xor_sync(0xffffffffu, send, o);
         }
-#pragma unroll
-    for (int p = 0; p < A3_NP; ++p) {
-        const double s = block_sum(val[p], red);
-        if (threadIdx.x == 0) part[d.part_off + (int64_t)lb * A3_NP + p] = s;
+    }
+    val[0] += __shfl_xor_sync(0xffffffffu, val[0], 1);
+    if (!(lane & 1)) red[wid][((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1)] = val[0];
+    __syncthreads();
+    if (threadIdx.x < A3_NP) {
+        double t = 0.0;
+        for (int w = 0; w < T3 / 32; ++w) t += red[w][threadIdx.x];
+        part[d.part_off + (int64_t)lb * A3_NP + threadIdx.x] = t;
     }
 }
 
-// One block per realization: fixed-order sums of its partials, then A.
-__global__ void k3_a_hom_final(Grp g, const double* __restrict__ part, double* __restrict__ A,
-                               double* __restrict__ Af) {
-    __shared__ double red[32];
+// One block per realization, a warp per sum (in tile order), then A.
+__global__ void __launch_bounds__(512) k3_a_hom_final(Grp g, const double* __restrict__ part,
+                                                      double* __restrict__ A, double* __restrict__ Af) {
+    __shared__ double s[A3_NP];
     const int un = g.first + blockIdx.x;
     const U3& d = g.desc[un];
     const int b = d.real;
-    const int tiles = (int)(((int64_t)d.n * d.n * d.n) / T3);
-    double s[A3_NP];
-#pragma unroll
-    for (int p = 0; p < A3_NP; ++p) {
-        double t = 0.0;
-        for (int k = threadIdx.x; k < tiles; k += blockDim.x) t += part[d.part_off + (int64_t)k * A3_NP + p];
-        s[p] = block_sum(t, red);
-    }
-    if (threadIdx.x != 0) return;
-    const double iv = d.inv_vol;
-    const int sym[3][3] = {{1, 2, 3}, {2, 4, 5}, {3, 5, 6}};
-    for (int x = 0; x < 3; ++x)
-        for (int y = 0; y < 3; ++y) {
-            A[9 * (int64_t)b + 3 * x + y] = s[sym[x][y]] * iv;
-            if (Af) Af[9 * (int64_t)b + 3 * x + y] = s[7 + 3 * x + y] * iv;
-        }
+    const int tiles = (int)(((int64_t)d.n * d.n * d.n) / (A3_PLANES * T3));
+    const int p = threadIdx.x >> 5;
+    const double t = warp_sum_array(part + d.part_off + p, tiles, A3_NP);
+    if ((threadIdx.x & 31) == 0) s[p] = t * d.inv_vol;
+    __syncthreads();
+    if (threadIdx.x >= 9) return;
+    const int x = threadIdx.x / 3, y = threadIdx.x % 3;
+    const int lo = min(x, y), hi = max(x, y);
+    A[9 * (int64_t)b + threadIdx.x] = s[1 + (lo == 0 ? hi : lo + hi + 1)];   // 11 12 13 22 23 33
+    if (Af) Af[9 * (int64_t)b + threadIdx.x] = s[7 + threadIdx.x];
 }
 
 // ------------------------------------- layout: ABI triples <-> unit pairs --
@@ -1793,12 +1817,13 @@ rve_status rve3_a_hom(const rve_realization* r, int32_t batch, const uint8_t* ma
     const Cells3T<double> cs{mask, coef};
     for (const Group3& g : p.groups) {
         const int per = (int)(nodes_of(g) / T3);
-        const Grp gr = W.grp(g, per, true);
+        const int tiles = per / A3_PLANES;
+        const Grp gr = W.grp(g, tiles, true);
         if (scheme == RVE_Q1_LUMPED)
-            k3_a_hom_part<1><<<nblocks(g, per, true), T3, 0, s>>>(gr, cs, u, W.part());
+            k3_a_hom_part<1><<<nblocks(g, tiles, true), T3, 0, s>>>(gr, cs, u, W.part());
         else
-            k3_a_hom_part<0><<<nblocks(g, per, true), T3, 0, s>>>(gr, cs, u, W.part());
-        k3_a_hom_final<<<g.count / 2, 256, 0, s>>>(W.grp(g, 1, true), W.part(), A, A_flux);
+            k3_a_hom_part<0><<<nblocks(g, tiles, true), T3, 0, s>>>(gr, cs, u, W.part());
+        k3_a_hom_final<<<g.count / 2, 32 * A3_NP, 0, s>>>(W.grp(g, 1, true), W.part(), A, A_flux);
         note_launch(2);
     }
     return cudaGetLastError() == cudaSuccess ? RVE_OK : RVE_ECUDA;
