@@ -664,15 +664,78 @@ __global__ void __launch_bounds__(T3) k3_rhs(Grp g, Cells3T<double> cs, double2*
 // r.z, and so beta, comes from the z solve one pass earlier.  Before, the pass
 // stored z and read r for r.z, a launch formed p = z + beta p, and e += alpha p
 // read p beside the residual's update: 177 bytes per node and step in FP32,
-// 145 now; 15 realizations of 64^3 37.4 -> 33.4 ms.
+// 145 now; 15 realizations of 64^3 37.4 -> 33.2 ms.
+// Double pairs are transformed in fixed point (rve_fixed.cuh, as the 2D rows
+// are), the block's lines all of them or, where one cannot be, all in FP64.
 template <typename T> __device__ __forceinline__ T alpha_of(const MixScal& s, int k);
 template <typename T> __device__ __forceinline__ T beta_of(const MixScal& s, int k);
+template <int LOG2N, int BS>
+__device__ __noinline__ void hartley_line_fp64(double2* w, double2* buf, int t, const double2* __restrict__ tw) {
+    constexpr int n = 1 << LOG2N, TL = n / 8;
+    double2 v[8];
+#pragma unroll
+    for (int m = 0; m < 8; ++m) v[m] = w[m];
+    fft_reg<FFT_TO_BOTH, LOG2N, BS>(v, buf, LOG2N, t, tw, true);
+#pragma unroll
+    for (int m = 0; m < 8; ++m) w[m] = hartley_pair(v[m], buf[pidx((n - (t + m * TL)) & (n - 1)) * BS]);
+}
+// w[m] = element t + m TL of line q -> of its Hartley transform; `ex` (shared):
+// two words per line of the block.
+template <int LOG2N, int BS>
+__device__ __forceinline__ void hartley_line(double2 (&w)[8], double2* buf, int q, int t, const Tables& tb,
+                                             unsigned* ex) {
+    constexpr int n = 1 << LOG2N, TL = n / 8, G = 256 / TL;
+    if (threadIdx.x < 2 * G) ex[threadIdx.x] = 0u;
+    unsigned hi = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+        hi = max(hi, max((unsigned)__double2hiint(w[m].x) & 0x7FFFFFFFu, (unsigned)__double2hiint(w[m].y) & 0x7FFFFFFFu));
+    if (hi == 0u) {   // zeros, or subnormals (which count as 1)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) hi |= (__double2loint(w[m].x) | __double2loint(w[m].y)) != 0;
+    }
+    __syncthreads();
+    atomicMax(ex + q, hi);
+    __syncthreads();
+    unsigned E = ex[q] == 0u ? 1023u : ex[q] >> 20;   // a line of zeros fits any unit
+    if (LOG2N >= 7 && fx_takes(E)) {
+        unsigned s = 0;
+#pragma unroll
+        for (int m = 0; m < 8; ++m)
+            s += fx_size((unsigned)__double2hiint(w[m].x), E) + fx_size((unsigned)__double2hiint(w[m].y), E);
+        atomicAdd(ex + G + q, s);
+    }
+    if (__syncthreads_and(fx_takes(E))) {
+        FxTw fx = fx_twiddles(tb, n);
+        fx.f = fx_schedule(LOG2N, ex[G + q]);
+        E -= fx.f.finer;
+        longlong2 f[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) f[m] = make_longlong2(fx_from(w[m].x, E), fx_from(w[m].y, E));
+        longlong2* fb = reinterpret_cast<longlong2*>(buf);
+        fft_reg<FFT_TO_BOTH, LOG2N, BS>(f, fb, LOG2N, t, fx, true);
+        const int e = (int)E - FX_BITS + fx_scale(LOG2N, fx.f) - 1;   // the pairs come doubled
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const longlong2 h = hartley_pair2(f[m], fb[pidx((n - (t + m * TL)) & (n - 1)) * BS]);
+            w[m] = make_double2(fx_to(h.x, e), fx_to(h.y, e));
+        }
+    } else {
+        double2 v[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) v[m] = w[m];
+        hartley_line_fp64<LOG2N, BS>(v, buf, t, twiddles<double2>(tb, n));
+#pragma unroll
+        for (int m = 0; m < 8; ++m) w[m] = v[m];
+    }
+}
 template <int LOG2N, int AXIS, bool STEP, typename V>
 __global__ void __launch_bounds__(256) k3_lines(Grp g, Tables tb, const V* src, V* dst,
                                                 typename ScalarOf<V>::T scale, V* __restrict__ e,
                                                 const MixScal* sc) {
     typedef typename ScalarOf<V>::T T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ unsigned ex[sizeof(V) == 16 ? 2 * 256 * 8 / (1 << LOG2N) : 1];
     int lb;
     const int u = unit_of(g, lb);
     const U3 d = g.desc[u];   // issued before the flag test
@@ -690,7 +753,8 @@ __global__ void __launch_bounds__(256) k3_lines(Grp g, Tables tb, const V* src, 
     V w[8];
 #pragma unroll
     for (int mm = 0; mm < 8; ++mm) w[mm] = src[base + (t + mm * TL) * stride];
-    fft_reg<FFT_TO_BOTH, LOG2N, BS>(w, buf, LOG2N, t, twiddles<V>(tb, n), true);
+    if constexpr (sizeof(V) == 16) hartley_line<LOG2N, BS>(w, buf, q, t, tb, ex);
+    else fft_reg<FFT_TO_BOTH, LOG2N, BS>(w, buf, LOG2N, t, twiddles<V>(tb, n), true);
     T ax = 0, ay = 0, bx = 0, by = 0;
     if (STEP) {
         ax = alpha_of<T>(sc[u], 0);
@@ -714,7 +778,8 @@ __global__ void __launch_bounds__(256) k3_lines(Grp g, Tables tb, const V* src, 
         for (int mm = 0; mm < 4; ++mm) {
             const int kx = t + (h + mm) * TL;
             const int64_t node = base + (int64_t)kx * stride;
-            const V hv = hartley_pair(w[h + mm], buf[pidx((n - kx) & (n - 1)) * BS]);
+            V hv = w[h + mm];   // FP64: transformed by hartley_line
+            if constexpr (sizeof(V) == 8) hv = hartley_pair(hv, buf[pidx((n - kx) & (n - 1)) * BS]);
             V o = mk<V>(scale * hv.x, scale * hv.y);
             if (STEP) {
                 e[node] = mk<V>(fma(ax, po[mm].x, eo[mm].x), fma(ay, po[mm].y, eo[mm].y));

@@ -67,3 +67,24 @@ def test_preconditioner_not_finite(n, bad):
     y, ref = (t.cpu().numpy().reshape(x.shape) for t in (y, ref))
     assert not np.isfinite(y[0, n // 2]).any()
     np.testing.assert_array_equal(y[1], ref[1])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [32, 64, 128])
+def test_preconditioner_lines_3d(n):
+    """Lines of the 3D transforms: zeros, spikes and magnitudes that leave the fixed-point path."""
+    from paper_1903_12227_gb300 import rve3
+    ds = [workloads.realization3(n // 8, 8, 10.0, 0, k) for k in range(2)]
+    g = np.random.default_rng(n)
+    x = g.standard_normal((2, n, n, n, 3))
+    x[0, ::3] = 0.0
+    x[0, 1, 1] *= 1e-290
+    x[1] = 0.0
+    x[1, n // 3, 2, [1, n - 2], :] = [[1.0, 0.0, 2.0], [-1.0, 3.0, 0.0]]
+    y = rve3.apply_precond(ds, torch.tensor(x.reshape(-1, 3), device="cuda"), delta=0.5)
+    y = y.cpu().numpy().reshape(x.shape)
+    lam = 4 * np.sin(np.pi * np.arange(n) / n) ** 2
+    sym = 5.5 * (lam[:, None, None] + lam[:, None] + lam) + 0.5
+    for k in range(2):   # as in 2D: |B^-1| |B| < 200
+        ref = np.fft.ifftn(np.fft.fftn(x[k], axes=(0, 1, 2)) / sym[..., None], axes=(0, 1, 2)).real
+        assert np.linalg.norm(y[k] - ref) <= 1e-12 * np.linalg.norm(ref)
