@@ -48,6 +48,11 @@ rve_solve_opts resolved_opts(const rve_solve_opts* o) {
     return r;
 }
 
+// The fused path's stencil pass in two launches (fused_P_body, fused_Q_tile).
+// Below 1024 a tile holds 6 rows or more (FP32 14 at 512) and the halo costs less than
+// p through memory.
+static bool split_pass(int n, const rve_solve_opts& o) { return n >= 1024 && o.path == RVE_PATH_FUSED; }
+
 // Tile geometry of one realization.  Row kernels use 256 threads, n/8 per
 // row, so a transform group is G = 2048/n rows.  An update block takes tU
 // rows; the stencil tile keeps tS + 2 padded rows in shared memory; column
@@ -90,6 +95,8 @@ static void default_tiles(int n, size_t vb, int blockC, const rve_solve_opts& o,
         }
         if (smem_of(4) <= budget) break;   // else: large grids, fewer and taller tiles
     }
+    // split passes: 32 products per thread and tile (FP32 sums stay that short)
+    if (split_pass(n, o)) t.tS = vb == 8 ? 8192 / n : 4096 / n;
     int ts_tuned = 0, bc_tuned = 0;
     if (tuned_tiles(n, o.precision, o.path == RVE_PATH_PERSISTENT ? 1 : 0, &ts_tuned, &bc_tuned))
         t.tS = ts_tuned;
@@ -125,6 +132,7 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
     p.words = 0;
     p.max_log2n = 5;
     p.smemS = p.smemU = p.smemC = 0;
+    p.split = false;
     int64_t maxnb = 0, total = 0;
     int maxn = 0;
     for (int b = 0; b < batch; ++b) {
@@ -198,7 +206,11 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
         maxnb = std::max<int64_t>(maxnb, ((int64_t)n * n) / 1024);
         const size_t vb = p.vbytes;
         const size_t seq = (size_t)seq_stride(n);
-        p.smemS = std::max(p.smemS, (size_t)(t.tS + 2) * seq * vb + (size_t)(t.tS + 1) * (n / 32) * 4);
+        // (split: two sets of row buffers; heights are bounded alike)
+        const size_t tile = (size_t)(t.tS + 2) * seq * vb + (size_t)(t.tS + 1) * (n / 32) * 4;
+        if (tile > MAX_SMEM) return RVE_EINVAL;
+        if (split_pass(n, o)) p.split = true;
+        p.smemS = std::max(p.smemS, split_pass(n, o) ? (size_t)2 * (2048 / n) * seq * vb : tile);
         // two sets of row buffers (one transform group each) for the update
         // pass's streaming; the preconditioner's row passes use the first
         p.smemU = std::max(p.smemU, (size_t)2 * std::min(t.tU, 2048 / n) * seq * vb);

@@ -13,7 +13,11 @@ namespace rve {
 // blocks still took 10 us a step at 4600 blocks, 2 us at one.)
 template <typename V, int SCHEME>
 __global__ void __launch_bounds__(256, sizeof(V) == 8 ? 3 : 2) k_fused_RS(const Ctx c, int which) {
-    fused_RS_tile<V, SCHEME>(c, blockIdx.x, which);
+    fused_RS_tile<V, SCHEME, true>(c, blockIdx.x, which);
+}
+template <typename V, int SCHEME>
+__global__ void __launch_bounds__(256, sizeof(V) == 8 ? 3 : 2) k_fused_Q(const Ctx c) {
+    fused_Q_tile<V, SCHEME>(c, blockIdx.x);
 }
 template <typename V>
 __global__ void __launch_bounds__(256, sizeof(V) == 8 ? 4 : 2) k_fused_U(const Ctx c) { fused_U_tile<V>(c, blockIdx.x); }
@@ -29,11 +33,15 @@ cudaError_t fused_step(const Plan& p, const Ctx& c, cudaStream_t s, cudaEvent_t*
         k_fused_RS<V, SCHEME><<<p.tilesS, 256, p.smemS, s>>>(c, DO_REFINE);
         cudaEventRecord(ev[1], s);
         k_fused_RS<V, SCHEME><<<p.tilesS, 256, p.smemS, s>>>(c, DO_STENCIL);
-        cudaEventRecord(ev[2], s);
         note_launch();
     } else {
         k_fused_RS<V, SCHEME><<<p.tilesS, 256, p.smemS, s>>>(c, DO_REFINE | DO_STENCIL);
     }
+    if (p.split) {
+        k_fused_Q<V, SCHEME><<<p.tilesS, 256, 0, s>>>(c);
+        note_launch();
+    }
+    if (ev) cudaEventRecord(ev[2], s);
     k_fused_U<V><<<p.tilesU, 256, p.smemU, s>>>(c);
     if (ev) cudaEventRecord(ev[3], s);
     k_fused_C<V><<<p.tilesC, p.blockC, p.smemC, s>>>(c);

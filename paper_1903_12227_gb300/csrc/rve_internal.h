@@ -67,6 +67,7 @@ struct Plan {
     std::vector<int32_t> startS, startU, startC, startA, startA2;
     int tilesS = 0, tilesU = 0, tilesC = 0, tilesA = 0, tilesA2 = 0;
     size_t smemS = 0, smemU = 0, smemC = 0;
+    bool split = false;             // some grid takes the stencil pass in two launches
     int cellsA = 1024;              // cells per FP64 A_hom tile
     int blockC = 512;               // threads of a column-solve block
     int persist_grid = 0;           // blocks of the persistent launch (0 = not prepared)

@@ -76,7 +76,7 @@ struct PersistArgs {
 // allocation inside the one persistent kernel.
 template <typename V, int SCHEME>
 __device__ __noinline__ void phase_RS(const Ctx& c, int t) {
-    fused_RS_tile<V, SCHEME>(c, t, DO_REFINE | DO_STENCIL);
+    fused_RS_tile<V, SCHEME, false>(c, t, DO_REFINE | DO_STENCIL);
 }
 template <typename V>
 __device__ __noinline__ void phase_U(const Ctx& c, int t) { fused_U_tile<V>(c, t); }

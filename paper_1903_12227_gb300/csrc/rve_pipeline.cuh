@@ -695,10 +695,213 @@ __device__ __forceinline__ void fused_S_body(const Ctx& c, int tile, int b, cons
     finish_S(c, b, s, false, sizeof(V) == 16 ? row_scale<SCHEME>() : 1.0);
 }
 
-// The refine or the stencil tile, by the realization's phase (`which`: 1
-// refine, 2 stencil, 3 both: the profiler times the two apart).
-enum { DO_REFINE = 1, DO_STENCIL = 2 };
+// The stencil pass of large grids (n >= 2^SPLIT_LOG2N, fused path) in two
+// launches.  A tile of whole rows holds few of them there (4 to 6), and the two
+// halo rows made their transforms 1.3 to 1.5 times the work at two blocks per
+// SM.  Instead the row half transforms and updates every row once and stores p,
+// and the stencil half (fused_Q_tile) reads p with its halo rows from L2: 56
+// bytes per node pair instead of 48, no halo transforms, five blocks per SM.
+// Per step: 2 x 2048^2 FP32 178 -> 142 us, 1024^2 FP64 130 -> 115 us.
+constexpr int SPLIT_LOG2N = 10;
+template <typename V, int LOG2N>
+__device__ __forceinline__ void fused_P_body(const Ctx& c, int tile, int b, const RState& s,
+                                             const RDesc& d, typename ScalarOf<V>::T* bsc,
+                                             unsigned* fxs) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    typedef typename ScalarOf<V>::T T;
+    const RowLayout<LOG2N> L(d.log2n);
+    const Sz<LOG2N>& z = L.z;
+    const int n = z.n;
+    const int r0 = (tile - c.startS[b]) * d.tS;
+    const int TR = min(d.tS, n - r0);
+    const int ng = (TR + L.G - 1) / L.G;
+    const V* Pold = static_cast<const V*>(s.parity ? c.P1 : c.P0);
+    V* Pnew = static_cast<V*>(s.parity ? c.P0 : c.P1);
+    V* X = static_cast<V*>(c.X);
+    const V* Tin = static_cast<const V*>(c.T);
+    {   // rows read after their transforms: asked for in L2 now
+        const unsigned rb = (unsigned)(n * sizeof(V));
+        const int k = threadIdx.x;
+        if (k < TR) prefetch_l2(Pold + node_at(d, z, r0 + k, 0), rb);
+        else if (k >= 64 && k < 64 + TR) prefetch_l2(X + node_at(d, z, r0 + k - 64, 0), rb);
+    }
+    if (threadIdx.x == 0) {
+        bsc[0] = (T)s.beta[0];
+        bsc[1] = (T)s.beta[1];
+        bsc[2] = (T)s.alpha[0];
+        bsc[3] = (T)s.alpha[1];
+    }
+    const int SEQ = seq_stride(n);
+    V* bufs = reinterpret_cast<V*>(smem_raw);   // two sets of L.G row buffers
+    auto prefetch = [&](int g) {   // zhat of group g into row buffer set g & 1
+        const int q = g * L.G + L.qq;
+        if (g < ng && q < TR) {
+            V* buf = bufs + ((g & 1) * L.G + L.qq) * SEQ;
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+                cp_async_v(buf + pidx(L.t + m * z.T), Tin + node_at(d, z, r0 + q, L.t + m * z.T));
+        }
+        cp_async_commit();
+    };
+    prefetch(0);
+    __syncthreads();
+    const T bx = bsc[0], by = bsc[1], alx = bsc[2], aly = bsc[3];
+    const V* tw = twiddles<V>(c.tb, n);
+    const FxTw fx = fx_twiddles(c.tb, n);
+    const TeamBar team(L.qq, z.T);
+    for (int g = 0; g < ng; ++g) {
+        const int q = g * L.G + L.qq;
+        const bool active = q < TR;
+        const int row = r0 + q;
+        prefetch(g + 1);   // free since the barrier at the end of group g - 1
+        cp_async_wait<1>();
+        team();
+        V* buf = bufs + ((g & 1) * L.G + (active ? L.qq : 0)) * SEQ;
+        V v[8];
+        if (active) {
+#pragma unroll
+            for (int m = 0; m < 8; ++m) v[m] = buf[pidx(L.t + m * z.T)];
+        }
+        hartley_row<LOG2N>(v, buf, L.t, tw, fx, active, fxs, team);
+        if (active) {
+#pragma unroll
+            for (int h = 0; h < 8; h += 4) {   // a half's loads before its stores
+                V po[4], xo[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const int64_t node = node_at(d, z, row, L.t + (h + m) * z.T);
+                    po[m] = Pold[node];
+                    xo[m] = X[node];
+                }
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const int64_t node = node_at(d, z, row, L.t + (h + m) * z.T);
+                    Pnew[node] = axpy2(v[h + m], bx, by, po[m]);
+                    X[node] = axpy2(xo[m], alx, aly, po[m]);
+                }
+            }
+        }
+        team();   // mirror reads of this row buffer are done
+    }
+    cp_async_wait<0>();
+}
+
+// The stencil half: q = A p on the tile's rows (FP64: K q, see StencilRow), p.q.
+// A thread walks down two columns (FP32) or one (FP64).
 template <typename V, int SCHEME>
+__device__ void fused_Q_tile(const Ctx& c, int tile) {
+    typedef typename ScalarOf<V>::T T;
+    __shared__ double red[64];
+    __shared__ T bsc[2];
+    __shared__ __align__(16) double rowtab[sizeof(V) == 16 ? ROW_TABLE : 2];
+    const int b = find_real(c.startS, c.batch, tile);
+    const RState& s = c.st[b];
+    if (s.phase != PH_ITER) return;
+    const RDesc d = c.desc[b];
+    if (d.log2n < SPLIT_LOG2N) return;
+    const int n = d.n, m = n - 1, lg = d.log2n;
+    const int r0 = (tile - c.startS[b]) * d.tS, r1 = min(r0 + d.tS, n);
+    const V* __restrict__ P = static_cast<const V*>(s.parity ? c.P0 : c.P1) + d.node_off;
+    V* __restrict__ Q = static_cast<V*>(c.Q) + d.node_off;
+    const uint32_t* __restrict__ mw = c.cs.coef ? nullptr : c.cs.mask + d.word_off;
+    const double* __restrict__ cf = c.cs.coef ? c.cs.coef + d.node_off : nullptr;
+    if (sizeof(V) == 16) {
+        if (mw) fill_row_table<SCHEME>(rowtab, d.a_matrix, d.a_incl);
+    } else if (threadIdx.x == 0) {
+        bsc[0] = (T)d.a_incl;
+        bsc[1] = (T)d.a_matrix;
+    }
+    __syncthreads();
+    DotAcc<T> ax, ay;
+    auto word = [&](int i, int jj) { return __ldg(mw + ((((int64_t)(i & m)) << lg) + jj >> 5)) >> (jj & 31); };
+    if constexpr (sizeof(V) == 16) {
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+            const int jm = (j - 1) & m, jp = (j + 1) & m;
+            auto at = [&](int i, int jj) { return __ldg(P + ((int64_t)(i & m) << lg) + jj); };
+            V u0 = at(r0 - 1, jm), u1 = at(r0 - 1, j), u2 = at(r0 - 1, jp);
+            V m0 = at(r0, jm), m1 = at(r0, j), m2 = at(r0, jp);
+            auto row = [&](const StencilRow& w, int i, const V& d0, const V& d1, const V& d2, auto doubled) {
+                const V q = apply_row<SCHEME, decltype(doubled)::value>(w, u0, u1, u2, m0, m1, m2, d0, d1, d2);
+                Q[((int64_t)i << lg) + j] = q;
+                ax.add(m1.x, q.x);
+                ay.add(m1.y, q.y);
+                u0 = m0; u1 = m1; u2 = m2;
+                m0 = d0; m1 = d1; m2 = d2;
+            };
+            if (mw) {
+                auto bits = [&](int i) -> unsigned { return (word(i, jm) & 1u) | ((word(i, j) & 1u) << 1); };
+                unsigned top = bits(r0 - 1);
+                for (int i = r0; i < r1; ++i) {
+                    const V d0 = at(i + 1, jm), d1 = at(i + 1, j), d2 = at(i + 1, jp);
+                    const unsigned bot = bits(i);
+                    row(table_row<SCHEME>(rowtab, top | (bot << 2)), i, d0, d1, d2, std::true_type());
+                    top = bot;
+                }
+            } else {
+                auto cell = [&](int i, int jj) { return __ldg(cf + ((int64_t)(i & m) << lg) + jj); };
+                RowWalk<SCHEME> walk(cell(r0 - 1, jm), cell(r0 - 1, j));
+                for (int i = r0; i < r1; ++i) {
+                    const V d0 = at(i + 1, jm), d1 = at(i + 1, j), d2 = at(i + 1, jp);
+                    row(walk.step(cell(i, jm), cell(i, j)), i, d0, d1, d2, std::false_type());
+                }
+            }
+        }
+    } else {
+        const float ai = bsc[0], am = bsc[1];
+        struct Row { V l, a, b, r; };     // p at j - 1, j, j + 1, j + 2
+        struct Cel { float l, a, b; };    // cells j - 1, j, j + 1
+        for (int j = 2 * threadIdx.x; j < n; j += 2 * blockDim.x) {
+            const int jm = (j - 1) & m, jp = (j + 2) & m;
+            auto prow = [&](int i) -> Row {
+                const V* p = P + ((int64_t)(i & m) << lg);
+                const float4 v = __ldg(reinterpret_cast<const float4*>(p + j));
+                return Row{__ldg(p + jm), make_float2(v.x, v.y), make_float2(v.z, v.w), __ldg(p + jp)};
+            };
+            auto crow = [&](int i) -> Cel {
+                if (mw) {
+                    const unsigned w = word(i, j), l = (j & 31) ? word(i, j - 1) : word(i, jm);
+                    return Cel{(l & 1u) ? ai : am, (w & 1u) ? ai : am, (w & 2u) ? ai : am};
+                }
+                const double* p = cf + ((int64_t)(i & m) << lg);
+                return Cel{(float)__ldg(p + jm), (float)__ldg(p + j), (float)__ldg(p + j + 1)};
+            };
+            Row u = prow(r0 - 1), v = prow(r0), ahead = prow(r0 + 1);
+            Cel t = crow(r0 - 1), o = crow(r0);
+#pragma unroll 2
+            for (int i = r0; i < r1; ++i) {
+                const Row dn = ahead;
+                ahead = prow(i + 2);
+                const Cel on = crow(i + 1);
+                const V q0 = stencil_apply<SCHEME, V>(CellsT<float>{t.l, t.a, o.l, o.a}, u.l, u.a, u.b, v.l, v.a,
+                                                      v.b, dn.l, dn.a, dn.b);
+                const V q1 = stencil_apply<SCHEME, V>(CellsT<float>{t.a, t.b, o.a, o.b}, u.a, u.b, u.r, v.a, v.b,
+                                                      v.r, dn.a, dn.b, dn.r);
+                *reinterpret_cast<float4*>(Q + ((int64_t)i << lg) + j) = make_float4(q0.x, q0.y, q1.x, q1.y);
+                ax.add(v.a.x, q0.x);
+                ay.add(v.a.y, q0.y);
+                ax.add(v.b.x, q1.x);
+                ay.add(v.b.y, q1.y);
+                u = v;
+                v = dn;
+                t = o;
+                o = on;
+            }
+        }
+    }
+    double sx = 0.0, sy = 0.0;
+    block_sum2(ax, ay, red, sx, sy);
+    if (threadIdx.x == 0) {
+        c.partS[2 * (int64_t)tile] = sx;
+        c.partS[2 * (int64_t)tile + 1] = sy;
+    }
+    finish_S(c, b, s, false, sizeof(V) == 16 ? row_scale<SCHEME>() : 1.0);
+}
+
+// The refine or the stencil tile, by the realization's phase (`which`: 1
+// refine, 2 stencil, 3 both: the profiler times the two apart).  SPLIT: the
+// row half of the stencil on large grids.
+enum { DO_REFINE = 1, DO_STENCIL = 2 };
+template <typename V, int SCHEME, bool SPLIT>
 __device__ void fused_RS_tile(const Ctx& c, int tile, int which) {
     __shared__ double red[64];   // block_sum2 scratch
     __shared__ unsigned fxs[8];  // row teams' reductions
@@ -712,7 +915,10 @@ __device__ void fused_RS_tile(const Ctx& c, int tile, int which) {
         refine_tile<V, SCHEME>(c, tile, b, s, d);
         return;
     }
-    dispatch_size(d.log2n, [&]<int LG>() { fused_S_body<V, SCHEME, LG>(c, tile, b, s, d, red, bsc, fxs, rowtab); });
+    dispatch_size(d.log2n, [&]<int LG>() {
+        if constexpr (SPLIT && LG >= SPLIT_LOG2N) fused_P_body<V, LG>(c, tile, b, s, d, bsc, fxs);
+        else fused_S_body<V, SCHEME, LG>(c, tile, b, s, d, red, bsc, fxs, rowtab);
+    });
 }
 
 // ----------------------------------------------------------- U kernel --
