@@ -180,7 +180,7 @@ def per_entry_error(A, ref):
 
 
 # Thread instructions per node of the double-word true-residual pass
-# (k_fused_R): ncu instruction count of a refining launch divided by its
+# (the refine half of k_fused_RS): ncu instruction count of a refining launch divided by its
 # nodes, for the first refinement of a solve (r = f) and the later ones
 # (profiles/k_fused_R_refine_plain_L32_32copies.md).
 REFINE_INST_PER_NODE = 485.4
@@ -535,11 +535,11 @@ CUBES_DESC = ("L=4, h=1/16 (64^3 nodes, 262144 unknowns per corrector), contrast
               "cubes (density 0.7), PCG tol 1e-10 on the true residual, 3x3 A_hom")
 # Algorithmic bytes per unit-node (a unit = one corrector pair of a
 # realization) of one launch of each 3D kernel kind in the mixed solve:
-# FP32 stencil 17 (x, cells, y); line pass 18 on average (16, the last of
-# four also reads r); z solve 16; vector steps 36 on average (axpy 48, xpby
-# 24); true residual in double words 81 (the split of u into double words:
+# FP32 stencil 17 (x, cells, y); line pass 22 on average (16, the last of
+# four 40: z, p, e in, p, e out); z solve 16; residual update 24 (r, q in, r
+# out); true residual in double words 81 (the split of u into double words:
 # u in, 16-byte words out; the residual pass: words, f, cells in, r out).
-CUBES_BYTES = {"stiffness": 17.0, "lines": 18.0, "zsolve": 16.0, "vector": 36.0, "scalar": 0.0,
+CUBES_BYTES = {"stiffness": 17.0, "lines": 22.0, "zsolve": 16.0, "vector": 24.0, "scalar": 0.0,
                "resid64": 81.0}
 
 
@@ -643,9 +643,9 @@ def run_cubes(args):
         return per_launch, avg_s, per_launch / avg_s / 1e9
 
     # unit-node counts per kind: one stencil, four line passes, one z solve,
-    # two vector launches per unit CG step
+    # one vector launch per unit CG step
     per_kind_nodes = {"stiffness": unit_steps * n3, "lines": 4 * unit_steps * n3,
-                      "zsolve": unit_steps * n3, "vector": 2 * unit_steps * n3, "scalar": 0,
+                      "zsolve": unit_steps * n3, "vector": unit_steps * n3, "scalar": 0,
                       "resid64": sum(max(d["refinements"] - 2, 0) for d in info_d) * n3}
     dom = max(("stiffness", "lines", "zsolve", "vector"), key=lambda k: prof[k][0])
     bpl, avg_s, achieved = rate(dom, per_kind_nodes[dom])

@@ -240,16 +240,15 @@ def dos_study(Ls=(4, 8), N=20, lam=0.5, alpha=0.25, m0=8, eta=0.05, K=512, vecto
 
 # Algorithmic bytes per node of one launch of each 3D kernel kind: the
 # stencil reads x (a pair, 16 B) and the cell byte and writes y (16 B); a
-# line pass reads and writes a pair (the last one also reads r: 48 B, so
-# 36 B on average over the four passes); the z solve reads and writes a
-# pair; the CG vector steps of one iteration move 144 B (u, r, p, q read and
-# u, r written; z, p read and p written) over two launches; the scalar
-# launches move nothing; the FP64 true residual reads u, f and the cells and
-# writes r (49 B).  FP32 vectors (the mixed path's cycles) halve the vector
-# bytes.
-CUBE_BYTES = {"stiffness": 33.0, "lines": 36.0, "zsolve": 32.0, "vector": 72.0, "scalar": 0.0,
+# line pass reads and writes a pair (the step's last one reads z, p and e and
+# writes p and e: 80 B, so 44 B on average over the four passes); the z solve
+# reads and writes a pair; the residual's update reads r and q and writes r;
+# the scalar launches move nothing; the FP64 true residual reads u, f and the
+# cells and writes r (49 B).  FP32 vectors (the mixed path's cycles) halve the
+# vector bytes.
+CUBE_BYTES = {"stiffness": 33.0, "lines": 44.0, "zsolve": 32.0, "vector": 48.0, "scalar": 0.0,
               "resid64": 49.0}
-CUBE_BYTES_FP32 = {"stiffness": 17.0, "lines": 18.0, "zsolve": 16.0, "vector": 36.0,
+CUBE_BYTES_FP32 = {"stiffness": 17.0, "lines": 22.0, "zsolve": 16.0, "vector": 24.0,
                    "scalar": 0.0, "resid64": 49.0}
 
 
@@ -386,7 +385,7 @@ def kernel_rates(L=32, m0=16, batch=64, K=64, reps=10) -> list:
 
 
 def refine_rate(L=32, m0=16, copies=32) -> dict:
-    """The double-word true-residual pass (k_fused_R) of the mixed solver on
+    """The double-word true-residual pass (refine half of k_fused_RS) of the mixed solver on
     `copies` copies of one realization, so that every refining launch works
     on all of them at once: its CUDA-event time per launch over one solve
     (idle launches of the iteration steps included) from the library's
@@ -405,7 +404,7 @@ def refine_rate(L=32, m0=16, copies=32) -> dict:
     prof = rve.profile_read()["refine"]
     rve.profile_enable(False)
     d = rve.info_to_dicts(info, copies)[0]
-    return {"kernel": "k_fused_R (double-word true residual, mixed solver)",
+    return {"kernel": "k_fused_RS, refine half (double-word true residual, mixed solver)",
             "nodes": (L * m0) ** 2 * copies, "launches": prof["launches"],
             "refining_launches": d["refinements"], "steps": d["steps"],
             "ms_total": prof["ms"], "us_per_launch": 1e3 * prof["ms"] / max(prof["launches"], 1)}

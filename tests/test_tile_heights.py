@@ -29,3 +29,24 @@ def test_lone_and_batched_solves(n, count, scheme, precision):
         m = mask[k * words:(k + 1) * words]
         v, _ = rve.solve(ds[k:k + 1], mask=m, opts=opts)
         assert torch.equal(v, u[k * n * n:(k + 1) * n * n])
+
+
+@pytest.mark.parametrize("precision", [rve.FP64, rve.MIXED])
+@pytest.mark.parametrize("scheme", [rve.CONSISTENT, rve.LUMPED])
+@pytest.mark.parametrize("n", [512, 1024, 2048])
+def test_explicit_cells_equal_mask(n, scheme, precision):
+    """The stencil passes (one launch, and two from 1024 on) on explicit cells and on the mask."""
+    ds = workloads.batch(n // 8, 8, 10.0, 6, 1)
+    opts = rve.make_opts(scheme=scheme, precision=precision, tol=1e-10)
+    mask = rve.gen_field(ds)
+    coef = rve.coef_from_mask(ds, mask)
+    u, info = rve.solve(ds, mask=mask, opts=opts)
+    v, info2 = rve.solve(ds, coef=coef, opts=opts)
+    assert all(i["status"] == rve.RVE_OK for t in (info, info2) for i in rve.info_to_dicts(t, 1))
+    if precision == rve.MIXED:   # the same arithmetic on the same values
+        assert torch.equal(u, v)
+    A = rve.a_hom(ds, u, mask=mask, scheme=scheme)
+    B = rve.a_hom(ds, v, coef=coef, scheme=scheme)
+    # two answers to one tolerance: the energies differ by its square times the
+    # condition number, far below 1e-10 of them
+    assert float((A - B).abs().max()) <= 1e-10 * float(A.abs().max())
