@@ -1030,9 +1030,10 @@ constexpr int MAX_STALL = 4;
 
 // The scalar steps: one block per unit reduces the unit's partial pairs (n^3
 // >> pshift of them: one per block of the kernel that wrote them) in a fixed
-// order (per-thread strided sums, then the block tree) and thread 0 applies
-// `what`.  `tfac`: the cycle target is max(tfac tol |f| /
-// |r64|, inner_tol).
+// order (four warps per component, per-thread strided sums, then the warp tree)
+// and threads 0 and 1 apply `what`, one component each: FP64 square roots and
+// divisions cost about a microsecond each.  `tfac`: the cycle target is
+// max(tfac tol |f| / |r64|, inner_tol).
 struct ScalArgs {
     double tol, inner_tol, tfac;
     int max_iter;
@@ -1041,94 +1042,124 @@ __global__ void __launch_bounds__(256) k3_scalar(int first, const U3* __restrict
                                                  MixScal* scs,
                                                  const double* __restrict__ part, int what,
                                                  int pshift, ScalArgs a) {
-    __shared__ double red[32];
+    __shared__ double red[8];
     const int u = first + blockIdx.x;
     MixScal* sc = scs + u;
     const U3& d = desc[u];
     if (what != M_FNORM && what != M_REFINE && sc->done) return;
     if (what == M_REFINE && sc->outer_done) return;
     const int nb = (int)(((int64_t)d.n * d.n * d.n) >> pshift);   // partial pairs written
-    const double* pp = part + d.part_off;
-    double tx = 0.0, ty = 0.0;
-    for (int k = threadIdx.x; k < nb; k += blockDim.x) {
-        tx += pp[2 * k];
-        ty += pp[2 * k + 1];
-    }
-    const double sx = block_sum(tx, red);
-    const double sy = block_sum(ty, red);
-    if (threadIdx.x != 0) return;
-    const double v[2] = {sx, sy};
+    const double* pp = part + d.part_off + (threadIdx.x >> 7);
+    double t = 0.0;
+    for (int j = threadIdx.x & 127; j < nb; j += 128) t += pp[2 * j];
+    t = warp_sum(t);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x >= 2) return;
+    const int k = threadIdx.x;
+    const double v = (red[4 * k] + red[4 * k + 1]) + (red[4 * k + 2] + red[4 * k + 3]);
+    auto both = [](bool x) { return __all_sync(3u, x) != 0; };
+    int status = RVE_OK;   // of this component, where the step sets one
+    bool open;
     switch (what) {
-        case M_FNORM:
-            for (int k = 0; k < 2; ++k) {
-                sc->fnorm[k] = sqrt(v[k]);
-                sc->cdone[k] = !(v[k] > 0.0);
-                sc->active[k] = 0;
-                sc->iters[k] = 0;
-                sc->stall[k] = 0;
-                sc->relres[k] = 0.0;
-                sc->rn_prev[k] = sc->fnorm[k];
+        case M_FNORM: {
+            const double fn = sqrt(v);
+            const bool none = !(v > 0.0);
+            sc->fnorm[k] = fn;
+            sc->cdone[k] = none;
+            sc->active[k] = 0;
+            sc->iters[k] = 0;
+            sc->stall[k] = 0;
+            sc->relres[k] = 0.0;
+            sc->rn_prev[k] = fn;
+            const bool all = both(none);
+            if (k == 0) {
+                sc->refinements = 0;
+                sc->status = RVE_OK;
+                sc->done = 1;
+                sc->outer_done = all;
             }
-            sc->refinements = 0;
-            sc->status = RVE_OK;
-            sc->done = 1;
-            sc->outer_done = sc->cdone[0] && sc->cdone[1];
             break;
-        case M_REFINE:
-            sc->refinements += 1;
-            for (int k = 0; k < 2; ++k) {
-                sc->active[k] = 0;
-                sc->alpha[k] = sc->beta[k] = 0.0;
-                sc->alpha_f[k] = sc->beta_f[k] = 0.f;
-                sc->inv_s_f[k] = 0.f;
-                if (sc->cdone[k]) continue;
-                const double rn = sqrt(v[k]);
+        }
+        case M_REFINE: {
+            const int refs = sc->refinements + 1;
+            __syncwarp(3u);
+            sc->alpha[k] = sc->beta[k] = 0.0;
+            sc->alpha_f[k] = sc->beta_f[k] = 0.f;
+            sc->inv_s_f[k] = 0.f;
+            bool done = sc->cdone[k] != 0;
+            open = false;
+            if (!done) {
+                const double rn = sqrt(v);
                 sc->relres[k] = rn / sc->fnorm[k];
-                if (!isfinite(rn)) { sc->status = RVE_ENAN; sc->cdone[k] = 1; continue; }
-                if (rn <= a.tol * sc->fnorm[k]) { sc->cdone[k] = 1; continue; }
-                sc->stall[k] = (rn > 0.1 * sc->rn_prev[k]) ? sc->stall[k] + 1 : 0;
-                if (sc->iters[k] >= a.max_iter || sc->refinements > MAX_REFINE ||
-                    sc->stall[k] >= MAX_STALL) {
-                    sc->status = RVE_ENOCONV;
-                    sc->cdone[k] = 1;
-                    continue;
+                if (!isfinite(rn)) {
+                    status = RVE_ENAN;
+                    done = true;
+                } else if (rn <= a.tol * sc->fnorm[k]) {
+                    done = true;
+                } else {
+                    const int stall = (rn > 0.1 * sc->rn_prev[k]) ? sc->stall[k] + 1 : 0;
+                    sc->stall[k] = stall;
+                    if (sc->iters[k] >= a.max_iter || refs > MAX_REFINE || stall >= MAX_STALL) {
+                        status = RVE_ENOCONV;
+                        done = true;
+                    } else {
+                        sc->rn_prev[k] = rn;
+                        sc->s[k] = rn;
+                        sc->inv_s_f[k] = (float)(1.0 / rn);
+                        sc->target[k] = fmax(a.tfac * a.tol * sc->fnorm[k] / rn, a.inner_tol);
+                        open = true;
+                    }
                 }
-                sc->rn_prev[k] = rn;
-                sc->s[k] = rn;
-                sc->inv_s_f[k] = (float)(1.0 / rn);
-                sc->target[k] = fmax(a.tfac * a.tol * sc->fnorm[k] / rn, a.inner_tol);
-                sc->active[k] = 1;
             }
-            sc->outer_done = sc->cdone[0] && sc->cdone[1];
-            sc->done = !(sc->active[0] || sc->active[1]);
+            sc->cdone[k] = done;
+            sc->active[k] = open;
+            const bool all = both(done), idle = both(!open);
+            if (k == 0) {
+                sc->refinements = refs;
+                sc->outer_done = all;
+                sc->done = idle;
+            }
             break;
+        }
         case M_RHO0:
-            for (int k = 0; k < 2; ++k) sc->rho[k] = v[k];
+            sc->rho[k] = v;
             break;
-        case M_ALPHA:
-            for (int k = 0; k < 2; ++k) {
-                sc->alpha[k] = sc->active[k] ? sc->rho[k] / v[k] : 0.0;
-                sc->alpha_f[k] = (float)sc->alpha[k];
-                if (sc->active[k]) sc->iters[k] += 1;
+        case M_ALPHA: {
+            const bool act = sc->active[k] != 0;
+            const double al = act ? sc->rho[k] / v : 0.0;
+            sc->alpha[k] = al;
+            sc->alpha_f[k] = (float)al;
+            if (act) sc->iters[k] += 1;
+            break;
+        }
+        case M_CONV: {   // the cycle's residual starts at norm 1
+            open = sc->active[k] != 0;
+            if (open) {
+                const double rn = sqrt(v);
+                if (!isfinite(rn)) {
+                    status = RVE_ENAN;
+                    open = false;
+                    sc->cdone[k] = 1;
+                } else if (rn <= sc->target[k] || sc->iters[k] >= a.max_iter) {
+                    open = false;
+                }
+                sc->active[k] = open;
             }
+            const bool idle = both(!open);
+            if (k == 0) sc->done = idle;
             break;
-        case M_CONV:   // the cycle's residual starts at norm 1
-            for (int k = 0; k < 2; ++k) {
-                if (!sc->active[k]) continue;
-                const double rn = sqrt(v[k]);
-                if (!isfinite(rn)) { sc->status = RVE_ENAN; sc->active[k] = 0; sc->cdone[k] = 1; }
-                else if (rn <= sc->target[k] || sc->iters[k] >= a.max_iter) sc->active[k] = 0;
-            }
-            sc->done = !(sc->active[0] || sc->active[1]);
+        }
+        case M_BETA: {
+            const double be = sc->active[k] ? v / sc->rho[k] : 0.0;
+            sc->beta[k] = be;
+            sc->beta_f[k] = (float)be;
+            sc->rho[k] = v;
             break;
-        case M_BETA:
-            for (int k = 0; k < 2; ++k) {
-                sc->beta[k] = sc->active[k] ? v[k] / sc->rho[k] : 0.0;
-                sc->beta_f[k] = (float)sc->beta[k];
-                sc->rho[k] = v[k];
-            }
-            break;
+        }
     }
+    const int st0 = __shfl_sync(3u, status, 0), st1 = __shfl_sync(3u, status, 1);
+    if (k == 0 && (st0 != RVE_OK || st1 != RVE_OK)) sc->status = st1 != RVE_OK ? st1 : st0;
 }
 
 // The step scalars in the cycle's precision.
