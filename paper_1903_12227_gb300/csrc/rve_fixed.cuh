@@ -24,8 +24,9 @@
 // Error (2-norm, against long double, n = 32 .. 2048): 0.33 to 0.57 of the
 // FP64 transform's for normal and smooth rows, at most 0.9 for spikes and
 // heavy tails.
-// Rows with an infinity or a NaN, and rows so small that a result could be
-// subnormal, take the FP64 transform (fx_takes).
+// Rows with an infinity or a NaN, rows so large that a result could overflow,
+// and rows so small that one could be subnormal, take the FP64 transform
+// (fx_takes).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -35,7 +36,10 @@ namespace rve {
 
 typedef long long fx_t;
 constexpr int FX_BITS = 57;       // the row's largest component is in [2^57, 2^58)
-constexpr unsigned FX_E_MIN = 128, FX_E_MAX = 2046;   // biased exponents taken
+// Biased exponents taken.  A component of the result has at most 13 more than
+// the row's largest (2048 elements of modulus below 2^1.5 times its binade, and
+// the rounding), and a double's largest is 2046.
+constexpr unsigned FX_E_MIN = 128, FX_E_MAX = 2046 - 13;
 
 // High and low word of v, the low one signed (v = h 2^32 + l).
 __host__ __device__ __forceinline__ void fx_split(fx_t v, int& h, int& l) {
