@@ -58,10 +58,11 @@ static bool split_pass(int n, const rve_solve_opts& o) { return n >= 1024 && o.p
 // rows; the stencil tile keeps tS + 2 padded rows in shared memory; column
 // blocks use blockC threads, n / col_seg_rows per column.
 //
-// The geometry follows from the grid size and the precision alone, never from
-// the rest of the batch: the dot products are summed tile by tile, so a
-// realization's result is the same bits alone and in any batch.  Stencil
-// tiles: the height with the least ceil(n / tS) blocks times a block's latency
+// The geometry follows from the grid size, the precision and the path alone,
+// never from the rest of the batch: the dot products are summed tile by tile, so
+// a realization's result is the same bits alone and in any batch.  (Tuned tables
+// excepted: the column width recorded for the batch's largest grid holds for
+// all of it.)  Stencil tiles: the height with the least ceil(n / tS) blocks times a block's latency
 // and transform groups (the halo rows are transformed twice); FP64, bound by
 // arithmetic, the lower of two within 15 %, so that few realizations spread
 // over more SMs.
@@ -105,6 +106,15 @@ static void default_tiles(int n, size_t vb, int blockC, const rve_solve_opts& o,
     t.tS = std::min(t.tS, n);
 }
 
+// Threads of a column block: a segment of up to 32 rows per thread in registers.
+// Mixed: 128 (3 % faster than 256 and 13 % faster than 512 on 512^2 grids,
+// measured), more where 128 would leave a block under eight columns, whose rows
+// are its memory accesses.  FP64: 128 (1024^2: 47 us a pass, 51 us at 256), at
+// least two columns.
+static int col_threads(int n, size_t vb) {
+    return vb == 8 ? (n > 1024 ? 512 : n > 512 ? 256 : 128) : (n > 1024 ? 256 : 128);
+}
+
 rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_opts* opts,
                      Plan& p, bool need_vectors) {
     if (!r || batch <= 0 || batch > (1 << 22)) return RVE_EINVAL;
@@ -145,21 +155,18 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
     // threads per block while that leaves under two blocks per SM
     p.cellsA = 1024;
     while (p.cellsA > 64 && total < (int64_t)p.cellsA * 304) p.cellsA /= 4;
-    // column blocks: a segment of up to 32 rows per thread in registers.
-    // Mixed: 128 threads (3 % faster than 256 and 13 % faster than 512 on
-    // 512^2 grids, measured), more where 128 would leave a block under eight
-    // columns, whose rows are its memory accesses.  FP64: 128 threads (1024^2:
-    // 47 us a pass, 51 us at 256), at least two columns
-    p.blockC = (p.vbytes == 8) ? (maxn > 1024 ? 512 : maxn > 512 ? 256 : 128) : (maxn > 1024 ? 256 : 128);
+    // column blocks of one width for the whole batch (0: col_threads by grid)
+    int blockC = 0;
     {
         int ts_tuned = 0, bc_tuned = 0;
         if (maxn > 0 && tuned_tiles(maxn, o.precision, o.path == RVE_PATH_PERSISTENT ? 1 : 0,
                                     &ts_tuned, &bc_tuned))
-            p.blockC = std::min(512, std::max(32, bc_tuned));   // a loaded table may hold anything
+            blockC = std::min(512, std::max(32, bc_tuned));   // a loaded table may hold anything
     }
-    if (o.path == RVE_PATH_PERSISTENT) p.blockC = 256;   // one block shape for all phases
+    if (o.path == RVE_PATH_PERSISTENT) blockC = 256;   // one block shape for all phases
     if (o.col_tile > 0 && o.path != RVE_PATH_PERSISTENT)
-        p.blockC = std::min(512, std::max(32, o.col_tile));
+        blockC = std::min(512, std::max(32, o.col_tile));
+    p.cols.clear();
     for (int b = 0; b < batch; ++b) {
         const rve_realization& x = r[b];
         if (x.L <= 0 || x.m0 <= 0) return RVE_EINVAL;
@@ -172,10 +179,11 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
             !(x.a_incl > 0.0))
             return RVE_EINVAL;
         Tiles t;
-        default_tiles(n, p.vbytes, p.blockC, o, t);
+        const int threadsC = blockC > 0 ? blockC : col_threads(n, p.vbytes);
+        default_tiles(n, p.vbytes, threadsC, o, t);
         const int segs = n / col_seg_rows(n, (int)p.vbytes);   // threads per column
         if (t.tS < 1 || t.tS > n || t.tC < 1 || !pow2(t.tC) || n % t.tC ||
-            t.tC * segs > p.blockC)
+            t.tC * segs > threadsC)
             return RVE_EINVAL;
         RDesc& d = p.desc[b];
         std::memset(&d, 0, sizeof(d));
@@ -217,7 +225,18 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
         // segment end / start values (2 per column segment) and the
         // singular column's sums (2 per segment); FP64: segment values, roots
         // and totals (tC <= 16 segs: within the same space), and those sums
-        p.smemC = std::max(p.smemC, (size_t)(2 * t.tC + 2) * segs * vb);
+        const size_t smemC = (size_t)(2 * t.tC + 2) * segs * vb;
+        p.smemC = std::max(p.smemC, smemC);
+        auto cl = std::find_if(p.cols.begin(), p.cols.end(),
+                               [&](const ColClass& c) { return c.threads == threadsC; });
+        if (cl == p.cols.end()) {
+            p.cols.emplace_back();
+            cl = p.cols.end() - 1;
+            cl->threads = threadsC;
+            cl->start.assign(batch + 1, 0);
+        }
+        cl->smem = std::max(cl->smem, smemC);
+        cl->start[b + 1] = n / t.tC;   // summed below
     }
     if (p.smemS > MAX_SMEM || p.smemU > MAX_SMEM || p.smemC > MAX_SMEM) return RVE_EINVAL;
     p.tilesS = p.startS[batch];
@@ -225,6 +244,10 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
     p.tilesC = p.startC[batch];
     p.tilesA = p.startA[batch];
     p.tilesA2 = p.startA2[batch];
+    for (ColClass& c : p.cols) {
+        for (int b = 0; b < batch; ++b) c.start[b + 1] += c.start[b];
+        c.tiles = c.start[batch];
+    }
     // workspace layout
     size_t off = 0;
     auto take = [&](size_t bytes) {
@@ -237,6 +260,8 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
     p.o_startS = take(sizeof(int32_t) * (batch + 1));
     p.o_startU = take(sizeof(int32_t) * (batch + 1));
     p.o_startC = take(sizeof(int32_t) * (batch + 1));
+    for (ColClass& c : p.cols)
+        c.o_start = p.cols.size() == 1 ? p.o_startC : take(sizeof(int32_t) * (batch + 1));
     p.o_startA = take(sizeof(int32_t) * (batch + 1));
     p.o_startA2 = take(sizeof(int32_t) * (batch + 1));
     p.o_tw64 = take(sizeof(double2) * tab);

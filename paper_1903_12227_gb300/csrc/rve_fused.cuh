@@ -22,8 +22,8 @@ __global__ void __launch_bounds__(256, sizeof(V) == 8 ? 3 : 2) k_fused_Q(const C
 template <typename V>
 __global__ void __launch_bounds__(256, sizeof(V) == 8 ? 4 : 2) k_fused_U(const Ctx c) { fused_U_tile<V>(c, blockIdx.x); }
 template <typename V>
-__global__ void __launch_bounds__(512) k_fused_C(const Ctx c) {
-    fused_C_tile<V>(c, blockIdx.x);
+__global__ void __launch_bounds__(512) k_fused_C(const Ctx c, const int32_t* __restrict__ start) {
+    fused_C_tile<V>(c, start, blockIdx.x);
 }
 
 template <typename V, int SCHEME>
@@ -44,12 +44,18 @@ cudaError_t fused_step(const Plan& p, const Ctx& c, cudaStream_t s, cudaEvent_t*
     if (ev) cudaEventRecord(ev[2], s);
     k_fused_U<V><<<p.tilesU, 256, p.smemU, s>>>(c);
     if (ev) cudaEventRecord(ev[3], s);
-    k_fused_C<V><<<p.tilesC, p.blockC, p.smemC, s>>>(c);
+    // a launch per block width: with one width for the batch, that of its largest
+    // grid, the sums of the smaller ones depended on their company.  The tail of
+    // the second launch costs batches that mix widths 2 to 4 % (one 2048^2 and 60
+    // 512^2 grids 30.5 -> 31.2 ms, with 300 of 64^2 13.0 -> 13.5 ms)
+    const char* w = reinterpret_cast<const char*>(c.startC) - p.o_startC;
+    for (const ColClass& k : p.cols)
+        k_fused_C<V><<<k.tiles, k.threads, k.smem, s>>>(c, reinterpret_cast<const int32_t*>(w + k.o_start));
     if (ev) cudaEventRecord(ev[4], s);
     const cudaError_t ce = launch_control(p, c, s);
     if (ce != cudaSuccess) return ce;
     if (ev) cudaEventRecord(ev[5], s);
-    note_launch(4);
+    note_launch(3 + (int)p.cols.size());
     return cudaGetLastError();
 }
 
@@ -124,7 +130,6 @@ cudaError_t precond_passes(const Plan& p, void* ws, double delta, const V* x, V*
     char* w = static_cast<char*>(ws);
     const RDesc* desc = reinterpret_cast<const RDesc*>(w + p.o_desc);
     const int32_t* startU = reinterpret_cast<const int32_t*>(w + p.o_startU);
-    const int32_t* startC = reinterpret_cast<const int32_t*>(w + p.o_startC);
     const Tables tb = tables_of(p, ws);
     cudaError_t e = cudaFuncSetAttribute(k_row_hartley<V>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smemU);
@@ -133,11 +138,17 @@ cudaError_t precond_passes(const Plan& p, void* ws, double delta, const V* x, V*
                                  (int)p.smemC);
     if (e != cudaSuccess) return e;
     const int u0 = p.startU[b_first], un = p.startU[b_first + b_count] - u0;
-    const int c0 = p.startC[b_first], cn = p.startC[b_first + b_count] - c0;
     k_row_hartley<V><<<un, 256, p.smemU, s>>>(desc, startU, p.batch, u0, tb, x, tmp);
-    k_col_hartley<V><<<cn, p.blockC, p.smemC, s>>>(desc, startC, p.batch, c0, tb, delta, tmp);
+    int launches = 2;
+    for (const ColClass& k : p.cols) {
+        const int c0 = k.start[b_first], cn = k.start[b_first + b_count] - c0;
+        if (cn == 0) continue;
+        k_col_hartley<V><<<cn, k.threads, k.smem, s>>>(desc, reinterpret_cast<const int32_t*>(w + k.o_start),
+                                                       p.batch, c0, tb, delta, tmp);
+        ++launches;
+    }
     k_row_hartley<V><<<un, 256, p.smemU, s>>>(desc, startU, p.batch, u0, tb, tmp, y);
-    note_launch(3);
+    note_launch(launches);
     return cudaGetLastError();
 }
 

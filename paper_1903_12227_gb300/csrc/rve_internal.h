@@ -53,6 +53,15 @@ struct Tiles {
     int tC;   // columns per column-transform block
 };
 
+// Grids of one block width of the column pass: a launch of their own, tiles
+// numbered from 0 over the batch's realizations of that width.
+struct ColClass {
+    int threads = 0, tiles = 0;
+    size_t smem = 0;
+    std::vector<int32_t> start;     // [batch + 1]
+    size_t o_start = 0;             // in the workspace (o_startC if the only class)
+};
+
 struct Plan {
     int batch = 0;
     int precision = RVE_FP64;
@@ -66,10 +75,10 @@ struct Plan {
     // a_hom_strip_rows(n) rows (mixed A_hom)
     std::vector<int32_t> startS, startU, startC, startA, startA2;
     int tilesS = 0, tilesU = 0, tilesC = 0, tilesA = 0, tilesA2 = 0;
-    size_t smemS = 0, smemU = 0, smemC = 0;
+    size_t smemS = 0, smemU = 0, smemC = 0;   // smemC: the largest of the classes
+    std::vector<ColClass> cols;
     bool split = false;             // some grid takes the stencil pass in two launches
     int cellsA = 1024;              // cells per FP64 A_hom tile
-    int blockC = 512;               // threads of a column-solve block
     int persist_grid = 0;           // blocks of the persistent launch (0 = not prepared)
     size_t persist_smem = 0;
     // workspace offsets (bytes)

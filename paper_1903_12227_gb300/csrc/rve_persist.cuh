@@ -81,7 +81,7 @@ __device__ __noinline__ void phase_RS(const Ctx& c, int t) {
 template <typename V>
 __device__ __noinline__ void phase_U(const Ctx& c, int t) { fused_U_tile<V>(c, t); }
 template <typename V>
-__device__ __noinline__ void phase_C(const Ctx& c, int t) { fused_C_tile<V>(c, t); }
+__device__ __noinline__ void phase_C(const Ctx& c, int t) { fused_C_tile<V>(c, c.startC, t); }
 
 template <typename V, int SCHEME>
 __global__ void __launch_bounds__(256, 2) k_persistent(const Ctx c, const PersistArgs a) {

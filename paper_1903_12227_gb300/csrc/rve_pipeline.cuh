@@ -1135,17 +1135,18 @@ __device__ void col_transform_tile(const V* in, V* out, const RDesc& d,
     });
 }
 
+// `start`: of the tiles of this launch (c.startC, or those of a ColClass).
 template <typename V>
-__device__ void fused_C_tile(const Ctx& c, int blk) {
+__device__ void fused_C_tile(const Ctx& c, const int32_t* __restrict__ start, int blk) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double red[64];   // block_sum2 scratch: 4 floats per warp (<= 32 warps)
-    const int b = find_real(c.startC, c.batch, blk);
+    const int b = find_real(start, c.batch, blk);
     if (c.st[b].phase == PH_DONE) return;
     const RDesc d = c.desc[b];
-    col_transform_tile<V>(static_cast<const V*>(c.R), static_cast<V*>(c.T), d,
-                          (blk - c.startC[b]) * d.tC,
+    const int tile = blk - start[b];
+    col_transform_tile<V>(static_cast<const V*>(c.R), static_cast<V*>(c.T), d, tile * d.tC,
                           reinterpret_cast<V*>(smem_raw), c.tb, c.delta, red,
-                          c.partC + 2 * (int64_t)blk);
+                          c.partC + 2 * (int64_t)(c.startC[b] + tile));
 }
 
 // ------------------------------------------------------ control kernel --

@@ -262,6 +262,9 @@ rve_status upload_plan(const Plan& p, void* ws, cudaStream_t s) {
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(w + p.o_startA2, p.startA2.data(), sizeof(int32_t) * (p.batch + 1),
                             cudaMemcpyHostToDevice, s);
+    for (size_t k = 0; p.cols.size() > 1 && k < p.cols.size() && e == cudaSuccess; ++k)
+        e = cudaMemcpyAsync(w + p.cols[k].o_start, p.cols[k].start.data(),
+                            sizeof(int32_t) * (p.batch + 1), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return RVE_ECUDA;
     return launch_tables(p, ws, s) == cudaSuccess ? RVE_OK : RVE_ECUDA;
 }
@@ -343,6 +346,9 @@ rve_status upload_descriptors(const Plan& p, void* ws, cudaStream_t s) {
     for (int k = 0; k < 5 && e == cudaSuccess; ++k)
         e = cudaMemcpyAsync(w + offs[k], tabs[k]->data(), sizeof(int32_t) * (p.batch + 1),
                             cudaMemcpyHostToDevice, s);
+    for (size_t k = 0; p.cols.size() > 1 && k < p.cols.size() && e == cudaSuccess; ++k)
+        e = cudaMemcpyAsync(w + p.cols[k].o_start, p.cols[k].start.data(),
+                            sizeof(int32_t) * (p.batch + 1), cudaMemcpyHostToDevice, s);
     return e == cudaSuccess ? RVE_OK : RVE_ECUDA;
 }
 
