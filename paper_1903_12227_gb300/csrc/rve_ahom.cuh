@@ -159,6 +159,12 @@ __device__ __forceinline__ void a_hom_tile(const RDesc& d, int64_t tile, CoefSrc
     a_hom_block_sums(acc, red, out);
 }
 
+// Cells of an FP64 tile: one to four per thread of 64 to 256, fewer on small
+// grids, so that one realization alone spreads over the chip.  By the grid's own
+// size: the tiles are summed one by one, and A_hom has to be the same bits alone
+// and in any batch.
+__host__ __device__ constexpr int a_hom_cells(int n) { return n <= 128 ? 64 : n <= 256 ? 256 : AHOM_TILE; }
+
 // Rows of a strip of a_hom_strip: min(n, AHOM_STRIP / n) rows of n cells.
 constexpr int AHOM_STRIP = 8192;
 __host__ __device__ constexpr int a_hom_strip_rows(int n) {

@@ -143,18 +143,13 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
     p.max_log2n = 5;
     p.smemS = p.smemU = p.smemC = 0;
     p.split = false;
-    int64_t maxnb = 0, total = 0;
+    int64_t maxnb = 0;
     int maxn = 0;
     for (int b = 0; b < batch; ++b) {
         const int64_t nn = (int64_t)r[b].L * r[b].m0;
         if (nn < MIN_N || nn > MAX_N) continue;   // rejected below
         maxn = std::max(maxn, (int)nn);
-        total += nn * nn;
     }
-    // FP64 A_hom: four cells per thread of a 256-thread block, fewer cells and
-    // threads per block while that leaves under two blocks per SM
-    p.cellsA = 1024;
-    while (p.cellsA > 64 && total < (int64_t)p.cellsA * 304) p.cellsA /= 4;
     // column blocks of one width for the whole batch (0: col_threads by grid)
     int blockC = 0;
     {
@@ -167,6 +162,7 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
     if (o.col_tile > 0 && o.path != RVE_PATH_PERSISTENT)
         blockC = std::min(512, std::max(32, o.col_tile));
     p.cols.clear();
+    p.threadsA = 64;
     for (int b = 0; b < batch; ++b) {
         const rve_realization& x = r[b];
         if (x.L <= 0 || x.m0 <= 0) return RVE_EINVAL;
@@ -209,7 +205,9 @@ rve_status make_plan(const rve_realization* r, int32_t batch, const rve_solve_op
         p.startS[b + 1] = p.startS[b] + (n + t.tS - 1) / t.tS;
         p.startU[b + 1] = p.startU[b] + n / t.tU;   // tU a power of two
         p.startC[b + 1] = p.startC[b] + n / t.tC;
-        p.startA[b + 1] = p.startA[b] + (int32_t)(((int64_t)n * n) / p.cellsA);
+        p.startA[b + 1] = p.startA[b] + (int32_t)(((int64_t)n * n) / a_hom_cells(n));
+        // (threads beyond a tile's cells add zeros)
+        p.threadsA = std::max(p.threadsA, std::min(256, a_hom_cells(n)));
         p.startA2[b + 1] = p.startA2[b] + n / a_hom_strip_rows(n);
         maxnb = std::max<int64_t>(maxnb, ((int64_t)n * n) / 1024);
         const size_t vb = p.vbytes;

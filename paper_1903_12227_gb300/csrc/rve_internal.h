@@ -71,14 +71,14 @@ struct Plan {
     int64_t nodes = 0, words = 0;
     int max_log2n = 0;
     std::vector<RDesc> desc;        // host copy
-    // startA: tiles of cellsA cells (FP64 A_hom); startA2: strips of
+    // startA: tiles of a_hom_cells(n) cells (FP64 A_hom); startA2: strips of
     // a_hom_strip_rows(n) rows (mixed A_hom)
     std::vector<int32_t> startS, startU, startC, startA, startA2;
     int tilesS = 0, tilesU = 0, tilesC = 0, tilesA = 0, tilesA2 = 0;
     size_t smemS = 0, smemU = 0, smemC = 0;   // smemC: the largest of the classes
     std::vector<ColClass> cols;
     bool split = false;             // some grid takes the stencil pass in two launches
-    int cellsA = 1024;              // cells per FP64 A_hom tile
+    int threadsA = 64;              // threads of an FP64 A_hom block
     int persist_grid = 0;           // blocks of the persistent launch (0 = not prepared)
     size_t persist_smem = 0;
     // workspace offsets (bytes)

@@ -483,12 +483,13 @@ __global__ void __launch_bounds__(256, 3)
 template <int SCHEME, bool FLUX>
 __global__ void __launch_bounds__(256) k_a_hom_part_dd(const RDesc* __restrict__ desc,
                                                        const int32_t* __restrict__ start, int batch,
-                                                       int cells, CoefSrc cs,
+                                                       CoefSrc cs,
                                                        const double2* __restrict__ u,
                                                        double* __restrict__ part) {
     __shared__ ddouble red[FLUX ? 32 * AHOM_NP : 32];
     const int b = find_real(start, batch, blockIdx.x);
     const RDesc d = desc[b];
+    const int cells = a_hom_cells(d.n);
     double* out = part + (int64_t)blockIdx.x * 2 * AHOM_NP;
     if (FLUX) a_hom_tile_dd<SCHEME>(d, blockIdx.x - start[b], cells, cs, u, red, out);
     else a_hom_tile_energy<SCHEME>(d, blockIdx.x - start[b], cells, cs, u, red, out);
@@ -695,10 +696,9 @@ cudaError_t launch_a_hom(const Plan& p, void* ws, const uint32_t* mask, const do
     const bool lumped = scheme == RVE_Q1_LUMPED;
     const int gf = (p.batch + 7) / 8;
     if (precision == RVE_FP64) {
-        const int threads = std::min(256, p.cellsA);
         auto parts = lumped ? (A_flux ? k_a_hom_part_dd<1, true> : k_a_hom_part_dd<1, false>)
                             : (A_flux ? k_a_hom_part_dd<0, true> : k_a_hom_part_dd<0, false>);
-        parts<<<p.tilesA, threads, 0, s>>>(desc, start, p.batch, p.cellsA, cs, uu, part);
+        parts<<<p.tilesA, p.threadsA, 0, s>>>(desc, start, p.batch, cs, uu, part);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         if (lumped) k_a_hom_final_dd<1><<<p.batch, 256, 0, s>>>(desc, start, part, A, A_lo, A_flux);

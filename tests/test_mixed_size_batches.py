@@ -55,3 +55,18 @@ def test_preconditioner(delta, dtype):
     y = rve.apply_precond(ds, x, delta=delta)
     for k in range(len(ds)):
         assert torch.equal(rve.apply_precond(ds[k:k + 1], x[node[k]:node[k + 1]], delta=delta), y[node[k]:node[k + 1]])
+
+
+@pytest.mark.parametrize("scheme", [rve.CONSISTENT, rve.LUMPED])
+@pytest.mark.parametrize("want_flux", [False, True])
+@pytest.mark.parametrize("sizes", [SIZES, (32,) * 700, (128,) * 40, (256, 512, 256)])
+def test_a_hom(sizes, want_flux, scheme):
+    ds, mask, node = _batch(sizes)
+    u = 0.01 * torch.randn(node[-1], 2, dtype=torch.float64, device="cuda",
+                           generator=torch.Generator(device="cuda").manual_seed(4))
+    kw = {"scheme": scheme, "want_lo": True, "want_flux": want_flux}
+    whole = rve.a_hom(ds, u, mask=mask, **kw)
+    for k in sorted({0, 1, len(ds) // 2, len(ds) - 1} | set(range(min(8, len(ds))))):
+        lone = rve.a_hom(ds[k:k + 1], u[node[k]:node[k + 1]], mask=mask[node[k] // 32:node[k + 1] // 32], **kw)
+        for a, b in zip(lone, whole):
+            assert torch.equal(a, b[k:k + 1]), (k, sizes[k])
