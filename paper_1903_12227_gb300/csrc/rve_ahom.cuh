@@ -225,43 +225,40 @@ __device__ __forceinline__ void a_hom_strip(const RDesc& d, int strip, CoefSrc c
     a_hom_block_sums(acc, red, out);
 }
 
-// The energy form alone in double-double arithmetic (the A_hom of FP64 solves;
-// a_hom_tile_dd below adds the flux form).  FP64 operations are what it costs:
-// differences of u across a cell and the added h are two TwoSums, left
-// unnormalised; the products of a cell are gathered as in a compensated dot
-// product (Ogita, Rump & Oishi's Dot2: TwoProd, TwoSum, the errors added up in
-// a double), and only a thread's sums are normalised.  The error is O(eps^2) of
-// the terms' size, 390 operations per cell instead of 1680; 1024^2 cells 2.81 ->
-// 0.90 ms.  Partials out[2k], out[2k+1] (k = 1, 2, 3) = (hi, lo) of E_11,
-// E_12, E_22, valid in thread 0; `red` holds 32 ddouble (shared).
-struct dd_sum {   // sum of unevaluated (p, c): errors in lo
-    double hi, lo;
-    __device__ __forceinline__ void add(double p, double c) {
-        const ddouble s = dd_two_sum(hi, p);
-        hi = s.hi;
-        lo = __dadd_rn(lo, __dadd_rn(s.lo, c));
-    }
-    // x y of unnormalised pairs
-    __device__ __forceinline__ void add_product(ddouble x, ddouble y) {
-        const double p = __dmul_rn(x.hi, y.hi);
-        add(p, __fma_rn(x.hi, y.lo, __fma_rn(x.lo, y.hi, __fma_rn(x.hi, y.hi, -p))));
-    }
-};
-template <int SCHEME>
-__device__ __forceinline__ void a_hom_tile_energy(const RDesc& d, int64_t tile, int cells, CoefSrc cs,
-                                                  const double2* __restrict__ u, ddouble* red,
-                                                  double* out) {
+// FP64 form of a_hom_tile: the cell sums in double-double arithmetic on the FP64
+// pipe, the energy form alone or (FLUX) both forms.  Differences of u across a
+// cell are exact (TwoSum), products and sums carry ~106 bits, so the only error
+// left in A_hom is that of the correctors themselves -- which enters the energy
+// form only quadratically (it is stationary at the exact solution).  FP64
+// operations are what it costs, so a cell's energies are formed in the sum /
+// difference basis of its corners, where K E is diagonal: with
+//   a = v10 + v11 - v00 - v01, b = v01 + v11 - v00 - v10, c = v00 + v11 - v01 - v10,
+//   K v^T E v' = (3 (aa' + bb') / 2 + cc'), lumped (aa' + bb') / 2 + cc',
+//   K xi_1^T E P u = 3 h a (lumped h a), K xi_2^T E P u = 3 h b
+// (a, b of xi_1, xi_2 are 2h): three products per energy instead of six.  Every
+// sum is renormalised: gathering a cell's products with their errors in one
+// plain double took 390 operations per cell instead of 470, but the error of
+// A + A_lo was 1.1 to 1.4 times as large (rms against 113 bits, n = 32; this
+// form's is that of the six products).  Calls of 1024^2: energy form 2.81 ms as
+// six products, 0.95 in that plain double, 1.08 now; with the flux form 2.90 ->
+// 1.39 ms (its eight sums were reduced by a butterfly each).
+// Partials out[2k], out[2k+1] = (hi, lo) of a_hom_tile's sums (k = 1, 2, 3 alone
+// without FLUX), the same bits with and without FLUX; `red` holds 8 x (FLUX ? 8 :
+// 4) ddouble (shared).
+template <int SCHEME, bool FLUX>
+__device__ __forceinline__ void a_hom_tile_dd(const RDesc& d, int64_t tile, int cells, CoefSrc cs,
+                                              const double2* __restrict__ u, ddouble* red,
+                                              double* out) {
+    constexpr int NP = FLUX ? AHOM_NP : 4;   // E_11, E_12, E_22, -; or all eight
+    constexpr int E0 = FLUX ? 1 : 0;         // E_11's place
     const double h = d.h;
     const int n = d.n;
     auto at = [&](int i, int j) {   // periodic node access
         return u[d.node_off + ((int64_t)(i & (n - 1)) << d.log2n) + (j & (n - 1))];
     };
-    auto diff = [](double a, double b) { return dd_two_sum(a, -b); };
-    auto diff_h = [](double a, double b, double c) -> ddouble {   // (a - b) + c
-        const ddouble s = dd_two_sum(a, -b), t = dd_two_sum(s.hi, c);
-        return {t.hi, __dadd_rn(s.lo, t.lo)};
-    };
-    dd_sum acc[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
+    ddouble acc[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) acc[k] = ddouble{0.0, 0.0};
     for (int t = threadIdx.x; t < cells; t += blockDim.x) {
         const int64_t cidx = tile * cells + t;
         const int i = (int)(cidx >> d.log2n), j = (int)(cidx & (n - 1));
@@ -273,151 +270,63 @@ __device__ __forceinline__ void a_hom_tile_energy(const RDesc& d, int64_t tile, 
             a = ((w >> (cidx & 31)) & 1u) ? d.a_incl : d.a_matrix;
         }
         const double2 r00 = at(i, j), r01 = at(i, j + 1), r10 = at(i + 1, j), r11 = at(i + 1, j + 1);
-        dd_sum e[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
-        // edges and diagonals of the cell, v_i = xi_i + u_i (see a_hom_cell)
-        auto pair = [&](ddouble v1, ddouble v2, double wgt) {
-            const ddouble w1 = dd_scale2(v1, wgt);
-            e[0].add_product(w1, v1);
-            e[1].add_product(w1, v2);
-            e[2].add_product(dd_scale2(v2, wgt), v2);
-        };
-        pair(diff(r01.x, r00.x), diff_h(r01.y, r00.y, h), 1.0);
-        pair(diff_h(r10.x, r00.x, h), diff(r10.y, r00.y), 1.0);
-        pair(diff_h(r11.x, r01.x, h), diff(r11.y, r01.y), 1.0);
-        pair(diff(r11.x, r10.x), diff_h(r11.y, r10.y, h), 1.0);
-        if (SCHEME == 0) {
-            pair(diff_h(r11.x, r00.x, h), diff_h(r11.y, r00.y, h), 2.0);
-            pair(diff_h(r10.x, r01.x, h), diff_h(r10.y, r01.y, -h), 2.0);
-        }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) acc[k].add_product(ddouble{e[k].hi, e[k].lo}, ddouble{a, 0.0});
-    }
-    // three sums over the warp in six additions per lane: halves, then quarters
-    // of the warp keep one sum each (lanes 0, 8, 16 end with E_11, E_12, E_22)
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    ddouble v[4];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) v[k] = dd_fast_two_sum(acc[k].hi, acc[k].lo);
-    v[3] = ddouble{0.0, 0.0};
-    auto other = [](ddouble x, int o) -> ddouble {
-        return {__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
-    };
-    const bool h16 = lane & 16, h8 = lane & 8;
-    const ddouble x0 = dd_add(h16 ? v[2] : v[0], other(h16 ? v[0] : v[2], 16));
-    const ddouble x1 = dd_add(h16 ? v[3] : v[1], other(h16 ? v[1] : v[3], 16));
-    ddouble x = dd_add(h8 ? x1 : x0, other(h8 ? x0 : x1, 8));
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) x = dd_add(x, other(x, o));
-    if ((lane & 7) == 0) red[wid * 4 + (lane >> 3)] = x;
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        ddouble s = red[threadIdx.x];
-        for (int w = 1; w < nw; ++w) s = dd_add(s, red[w * 4 + threadIdx.x]);
-        out[2 * (threadIdx.x + 1)] = s.hi;
-        out[2 * (threadIdx.x + 1) + 1] = s.lo;
-    }
-}
-
-// FP64 form of a_hom_tile, energy and flux: the same cell sums in
-// double-double arithmetic on the FP64 pipe.  Differences of u across a cell
-// are exact (TwoSum), products and sums carry ~106 bits, so the only error
-// left in A_hom is that of the correctors themselves -- which enters the
-// energy form only quadratically (it is stationary at the exact solution).
-// Partials out[2k], out[2k+1] = (hi, lo) of the same eight sums, valid in
-// thread 0; `red` holds 32 * AHOM_NP ddouble (shared).  Contains barriers.
-template <int SCHEME>
-__device__ __forceinline__ void a_hom_tile_dd(const RDesc& d, int64_t tile, int cells, CoefSrc cs,
-                                              const double2* __restrict__ u, ddouble* red,
-                                              double* out) {
-    const double h = d.h;
-    constexpr double Q = SCHEME == 0 ? 2.0 : 0.0;   // K |E| on the cell diagonals
-    const int n = d.n;
-    auto at = [&](int i, int j) {   // periodic node access
-        return u[d.node_off + ((int64_t)(i & (n - 1)) << d.log2n) + (j & (n - 1))];
-    };
-    ddouble acc[AHOM_NP];
-#pragma unroll
-    for (int k = 0; k < AHOM_NP; ++k) acc[k] = ddouble{0.0, 0.0};
-    const int64_t base = tile * cells;
-    for (int t = threadIdx.x; t < cells; t += blockDim.x) {
-        const int64_t cidx = base + t;
-        const int i = (int)(cidx >> d.log2n), j = (int)(cidx & (n - 1));
-        double a;
-        if (cs.coef) {
-            a = __ldg(cs.coef + d.node_off + cidx);
-        } else {
-            const uint32_t w = __ldg(cs.mask + d.word_off + (cidx >> 5));
-            a = ((w >> (cidx & 31)) & 1u) ? d.a_incl : d.a_matrix;
-        }
-        const double2 r00 = at(i, j), r01 = at(i, j + 1);
-        const double2 r10 = at(i + 1, j), r11 = at(i + 1, j + 1);
-        // exact u differences per corrector: 01-00, 10-00, 11-00, 10-01,
-        // 11-01, 11-10
-        ddouble D[2][6];
+        ddouble w[2][3];   // a, b, c of the correctors
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
             const double u00 = c ? r00.y : r00.x, u01 = c ? r01.y : r01.x;
             const double u10 = c ? r10.y : r10.x, u11 = c ? r11.y : r11.x;
-            D[c][0] = dd_sub(u01, u00);
-            D[c][1] = dd_sub(u10, u00);
-            D[c][2] = dd_sub(u11, u00);
-            D[c][3] = dd_sub(u10, u01);
-            D[c][4] = dd_sub(u11, u01);
-            D[c][5] = dd_sub(u11, u10);
+            const ddouble d0 = dd_sub(u10, u00), d1 = dd_sub(u11, u01);
+            w[c][0] = dd_add(d0, d1);
+            w[c][1] = dd_add(dd_sub(u01, u00), dd_sub(u11, u10));
+            w[c][2] = dd_add(d1, dd_neg(d0));
         }
-        // differences of v_i = xi_i + u_i (as in a_hom_tile)
-        ddouble V1[6], V2[6];
-        V1[0] = D[0][0];            V2[0] = dd_add(D[1][0], h);
-        V1[1] = dd_add(D[0][1], h); V2[1] = D[1][1];
-        V1[2] = dd_add(D[0][2], h); V2[2] = dd_add(D[1][2], h);
-        V1[3] = dd_add(D[0][3], h); V2[3] = dd_add(D[1][3], -h);
-        V1[4] = dd_add(D[0][4], h); V2[4] = D[1][4];
-        V1[5] = D[0][5];            V2[5] = dd_add(D[1][5], h);
-        ddouble e11{0.0, 0.0}, e12{0.0, 0.0}, e22{0.0, 0.0};
+        if (FLUX) {   // P_11, P_12, P_21, P_22 over 3h (lumped h)
+            acc[0] = dd_add(acc[0], a);
 #pragma unroll
-        for (int p = 0; p < 6; ++p) {
-            const double wgt = (p == 2 || p == 3) ? Q : 1.0;   // diagonals 00-11, 01-10
-            if (wgt == 0.0) continue;
-            e11 = dd_add(e11, dd_scale2(dd_mul(V1[p], V1[p]), wgt));
-            e12 = dd_add(e12, dd_scale2(dd_mul(V1[p], V2[p]), wgt));
-            e22 = dd_add(e22, dd_scale2(dd_mul(V2[p], V2[p]), wgt));
+            for (int k = 0; k < 4; ++k) acc[(4 + k) % NP] = dd_add(acc[(4 + k) % NP], dd_mul(w[k & 1][k >> 1], a));
         }
-        ddouble F[2][2];   // F[j][i] = xi_j^T (K E) P_c u_i, as in a_hom_tile
+        w[0][0] = dd_add(w[0][0], 2.0 * h);   // v_i = xi_i + u_i
+        w[1][1] = dd_add(w[1][1], 2.0 * h);
 #pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const ddouble qd11 = dd_scale2(D[c][2], Q), qd1001 = dd_scale2(D[c][3], Q);
-            F[0][c] = dd_mul(dd_add(dd_add(D[c][1], qd11), dd_add(qd1001, D[c][4])), h);
-            F[1][c] = dd_mul(dd_add(dd_add(D[c][0], qd11), dd_add(dd_neg(qd1001), D[c][5])), h);
+        for (int k = 0; k < 3; ++k) {
+            const int x = k == 2 ? 1 : 0, y = k == 0 ? 0 : 1;
+            const ddouble ab = dd_add(dd_mul(w[x][0], w[y][0]), dd_mul(w[x][1], w[y][1]));
+            const ddouble e = dd_add(SCHEME == 0 ? dd_mul(ab, 1.5) : dd_scale2(ab, 0.5), dd_mul(w[x][2], w[y][2]));
+            acc[E0 + k] = dd_add(acc[E0 + k], dd_mul(e, a));
         }
-        acc[0] = dd_add(acc[0], a);
-        acc[1] = dd_add(acc[1], dd_mul(e11, a));
-        acc[2] = dd_add(acc[2], dd_mul(e12, a));
-        acc[3] = dd_add(acc[3], dd_mul(e22, a));
-        acc[4] = dd_add(acc[4], dd_mul(F[0][0], a));
-        acc[5] = dd_add(acc[5], dd_mul(F[0][1], a));
-        acc[6] = dd_add(acc[6], dd_mul(F[1][0], a));
-        acc[7] = dd_add(acc[7], dd_mul(F[1][1], a));
     }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int nw = (blockDim.x + 31) >> 5;
+    if (FLUX) {
 #pragma unroll
-    for (int k = 0; k < AHOM_NP; ++k) {
-        const ddouble v = dd_warp_sum(acc[k]);
-        if (lane == 0) red[wid * AHOM_NP + k] = v;
+        for (int k = 4; k < NP; ++k) acc[k] = dd_mul(acc[k], SCHEME == 0 ? 3.0 * h : h);
     }
+    // the sums over the warp in NP + 1 or so additions per lane: at each of the
+    // first steps half of the lanes keep half of the sums
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    auto other = [](ddouble x, int o) -> ddouble {
+        return {__shfl_xor_sync(0xffffffffu, x.hi, o), __shfl_xor_sync(0xffffffffu, x.lo, o)};
+    };
+    int mine = 0;   // the sum that this lane ends with
+#pragma unroll
+    for (int o = 16, half = NP / 2; o > 0; o >>= 1, half >>= 1) {
+        if (half >= 1) {
+            const bool up = lane & o;
+#pragma unroll
+            for (int k = 0; k < half; ++k)
+                acc[k] = dd_add(up ? acc[k + half] : acc[k], other(up ? acc[k] : acc[k + half], o));
+            if (up) mine += half;
+        } else {
+            acc[0] = dd_add(acc[0], other(acc[0], o));
+        }
+    }
+    if ((lane & (32 / NP - 1)) == 0) red[wid * NP + mine] = acc[0];
     __syncthreads();
-    if (wid == 0) {
-#pragma unroll
-        for (int k = 0; k < AHOM_NP; ++k) {
-            ddouble v = lane < nw ? red[lane * AHOM_NP + k] : ddouble{0.0, 0.0};
-            v = dd_warp_sum(v);
-            if (lane == 0) {
-                out[2 * k] = v.hi;
-                out[2 * k + 1] = v.lo;
-            }
-        }
+    const int k = threadIdx.x + 1 - E0;   // of the eight
+    if (threadIdx.x < (FLUX ? AHOM_NP : 3)) {
+        ddouble s = red[threadIdx.x];
+        for (int w = 1; w < nw; ++w) s = dd_add(s, red[w * NP + threadIdx.x]);
+        out[2 * k] = s.hi;
+        out[2 * k + 1] = s.lo;
     }
-    __syncthreads();
 }
 
 // Energy and flux forms from the double-double tile partials (16 doubles per

@@ -486,13 +486,12 @@ __global__ void __launch_bounds__(256) k_a_hom_part_dd(const RDesc* __restrict__
                                                        CoefSrc cs,
                                                        const double2* __restrict__ u,
                                                        double* __restrict__ part) {
-    __shared__ ddouble red[FLUX ? 32 * AHOM_NP : 32];
+    __shared__ ddouble red[8 * (FLUX ? AHOM_NP : 4)];
     const int b = find_real(start, batch, blockIdx.x);
     const RDesc d = desc[b];
     const int cells = a_hom_cells(d.n);
     double* out = part + (int64_t)blockIdx.x * 2 * AHOM_NP;
-    if (FLUX) a_hom_tile_dd<SCHEME>(d, blockIdx.x - start[b], cells, cs, u, red, out);
-    else a_hom_tile_energy<SCHEME>(d, blockIdx.x - start[b], cells, cs, u, red, out);
+    a_hom_tile_dd<SCHEME, FLUX>(d, blockIdx.x - start[b], cells, cs, u, red, out);
 }
 
 template <int SCHEME>
