@@ -391,7 +391,7 @@ __global__ void __cluster_dims__(CHEB_CTAS, 1, 1) __launch_bounds__(32 * (CHEB_W
                 for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
                 const double nc = __shfl_down_sync(0xffffffffu, x, 2);   // lanes 0, 1
                 if (lane < 2) {
-                    double* mb = mu + ((int64_t)b * 2 + lane) * K;
+                    double* mb = mu + ((int64_t)ch.real[b] * 2 + lane) * K;
                     if (q == 0) { mu0 = x; mu1 = nc; }
                     if (2 * q < K) mb[2 * q] = q == 0 ? x : 2.0 * x - mu0;
                     if (2 * q + 1 < K) mb[2 * q + 1] = q == 0 ? nc : 2.0 * nc - mu1;
@@ -414,7 +414,7 @@ __global__ void k_cheb_moments(const __grid_constant__ DescChunk ch, const doubl
     for (int q = 0; q < 4; ++q) s[q] = warp_sum_array(part + (int64_t)t0 * 4 + q, nt, 4);
     if ((threadIdx.x & 31) != 0) return;
     for (int c = 0; c < 2; ++c) {
-        double* m = mu + ((int64_t)b * 2 + c) * K;
+        double* m = mu + ((int64_t)ch.real[b] * 2 + c) * K;
         const double cc = s[c], nc = s[2 + c];
         const double e = (k == 0) ? cc : 2.0 * cc - m[0];
         const double o = (k == 0) ? nc : 2.0 * nc - m[1];
@@ -532,6 +532,7 @@ static cudaError_t for_chunks(const Plan& p, UnitsFn units, LaunchFn fn) {
         ch.start[0] = 0;
         for (int k = 0; k < ch.count; ++k) {
             ch.d[k] = p.desc[b0 + k];
+            ch.real[k] = b0 + k;
             ch.start[k + 1] = ch.start[k] + (int32_t)units(ch.d[k]);
         }
         for (int k = ch.count + 1; k <= CHUNK; ++k) ch.start[k] = ch.start[ch.count];
@@ -636,22 +637,45 @@ cudaError_t launch_cheb(const Plan& p, void* ws, const uint32_t* mask, const dou
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_cheb_cluster<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e != cudaSuccess) return e;
-    return for_chunks(p, node_tiles, [&](const DescChunk& ch, int first_real) {
-        double* m = mu + (int64_t)first_real * 2 * K;
+    return for_chunks(p, node_tiles, [&](const DescChunk& all, int) {
+        // the form by each grid's own size (the two round differently)
+        DescChunk ch = all;
+        ch.count = 0;
         int maxn = 0;
-        int64_t nodes = 0;
-        for (int k = 0; k < ch.count; ++k) {
-            maxn = std::max(maxn, ch.d[k].n);
-            nodes += (int64_t)ch.d[k].n * ch.d[k].n;
+        for (int k = 0; k < all.count; ++k) {
+            if (all.d[k].n > CHEB_MAX_N) continue;
+            maxn = std::max(maxn, all.d[k].n);
+            ch.real[ch.count] = all.real[k];
+            ch.d[ch.count++] = all.d[k];
         }
-        if (maxn <= CHEB_MAX_N) {   // two vectors of a realization fit a cluster's shared memory
+        if (ch.count > 0) {   // two vectors of a realization fit a cluster's shared memory
             const size_t smem = 2 * sizeof(double2) * (size_t)maxn * maxn / CHEB_CTAS;
             auto kern = scheme == RVE_Q1_LUMPED ? k_cheb_cluster<1> : k_cheb_cluster<0>;
-            kern<<<ch.count * CHEB_CTAS, 32 * (CHEB_WARPS + 1), smem, s>>>(ch, cs, a0, a1, steps, K, v, m);
-            return cudaGetLastError();
+            kern<<<ch.count * CHEB_CTAS, 32 * (CHEB_WARPS + 1), smem, s>>>(ch, cs, a0, a1, steps, K, v, mu);
+            const cudaError_t ce = cudaGetLastError();
+            if (ce != cudaSuccess || ch.count == all.count) return ce;
         }
-        const cudaError_t ce = cudaMemcpyAsync(wb + ch.d[0].node_off, v + 2 * ch.d[0].node_off,
-                                               sizeof(double2) * (size_t)nodes, cudaMemcpyDeviceToDevice, s);   // w_0
+        ch.count = 0;
+        int64_t from = 0, to = 0;   // nodes of a run of realizations whose w_0 is still to copy
+        auto copy = [&]() -> cudaError_t {
+            if (from == to) return cudaSuccess;
+            return cudaMemcpyAsync(wb + from, v + 2 * from, sizeof(double2) * (size_t)(to - from),
+                                   cudaMemcpyDeviceToDevice, s);
+        };
+        for (int k = 0; k < all.count; ++k) {
+            const RDesc& d = all.d[k];
+            if (d.n <= CHEB_MAX_N) continue;
+            if (d.node_off != to) {
+                const cudaError_t ce = copy();
+                if (ce != cudaSuccess) return ce;
+                from = d.node_off;
+            }
+            to = d.node_off + (int64_t)d.n * d.n;
+            ch.start[ch.count + 1] = ch.start[ch.count] + (int32_t)node_tiles(d);
+            ch.real[ch.count] = all.real[k];
+            ch.d[ch.count++] = d;
+        }
+        const cudaError_t ce = copy();
         if (ce != cudaSuccess) return ce;
         const int g = ch.start[ch.count];
         double2* cur = wb;    // w_k
@@ -661,7 +685,7 @@ cudaError_t launch_cheb(const Plan& p, void* ws, const uint32_t* mask, const dou
                 k_cheb<1><<<g, NODE_TILE, 0, s>>>(ch, cs, a0, a1, k == 0, cur, oth, part);
             else
                 k_cheb<0><<<g, NODE_TILE, 0, s>>>(ch, cs, a0, a1, k == 0, cur, oth, part);
-            k_cheb_moments<<<(ch.count + 7) / 8, 256, 0, s>>>(ch, part, k, K, m);
+            k_cheb_moments<<<(ch.count + 7) / 8, 256, 0, s>>>(ch, part, k, K, mu);
             note_launch(2);
             const cudaError_t le = cudaGetLastError();
             if (le != cudaSuccess) return le;

@@ -70,3 +70,17 @@ def test_a_hom(sizes, want_flux, scheme):
         lone = rve.a_hom(ds[k:k + 1], u[node[k]:node[k + 1]], mask=mask[node[k] // 32:node[k + 1] // 32], **kw)
         for a, b in zip(lone, whole):
             assert torch.equal(a, b[k:k + 1]), (k, sizes[k])
+
+
+@pytest.mark.parametrize("scheme", [rve.CONSISTENT, rve.LUMPED])
+@pytest.mark.parametrize("sizes", [(64, 256, 32, 128, 512, 256, 64), (256, 256, 32), (32,) * 97 + (256, 64, 256)])
+def test_chebyshev_moments(sizes, scheme):
+    ds, mask, node = _batch(sizes, contrast=5.0)
+    K, hi = 33, 16 * 5.0
+    v = torch.randn(node[-1], 2, dtype=torch.float64, device="cuda",
+                    generator=torch.Generator(device="cuda").manual_seed(5))
+    mu = rve.cheb_moments(ds, v, K, 0.0, hi, mask=mask, scheme=scheme)
+    for k in sorted({0, 1, len(ds) // 2, len(ds) - 1} | set(range(max(0, len(ds) - 7), len(ds)))):
+        one = rve.cheb_moments(ds[k:k + 1], v[node[k]:node[k + 1]], K, 0.0, hi,
+                               mask=mask[node[k] // 32:node[k + 1] // 32], scheme=scheme)
+        assert torch.equal(one, mu[k:k + 1]), (k, sizes[k])
