@@ -21,9 +21,15 @@
 // Dense rows (c about n/4) need every bit of head room; rows of few large
 // elements (spectra) do not, and the unit they lose least by is a finer one.
 //
-// Error (2-norm, against long double, n = 32 .. 2048): 0.33 to 0.57 of the
-// FP64 transform's for normal and smooth rows, at most 0.9 for spikes and
-// heavy tails.
+// Error of one row (2-norm, against long double, as a part of that of the same
+// stages in double; tests/fixed_rows_host.cu): noise, smooth and dense rows 0.32 to
+// 0.72; spikes, heavy tails and spectra at most 0.65 up to n = 512, 0.94 at 1024,
+// 1.08 at 2048.  The worst rows found, a spike on noise of 1 to 5 % of it, reach
+// 1.4 and 1.5 at 1024 and 2048: three divisions where the row hardly grows.  (Giving
+// those bits back behind each product brings every row to 0.70 or less, and costs
+// a 1024^2 FP64 solve 2.6 %.)  Error of a whole B^-1 x (two row transforms and the
+// column pass, against 128-bit FFTs; noise, spikes, a spike on noise, smooth fields
+// and corrector loads, 512^2 to 2048^2): 0.75 to 0.99 of the FP64 form's.
 // Rows with an infinity or a NaN, rows so large that a result could overflow,
 // and rows so small that one could be subnormal, take the FP64 transform
 // (fx_takes).
