@@ -692,12 +692,13 @@ __device__ __forceinline__ void hartley_line(double2 (&w)[8], double2* buf, int 
         hi = max(hi, max((unsigned)__double2hiint(w[m].x) & 0x7FFFFFFFu, (unsigned)__double2hiint(w[m].y) & 0x7FFFFFFFu));
     if (hi == 0u) {   // zeros, or subnormals (which count as 1)
 #pragma unroll
-        for (int m = 0; m < 8; ++m) hi |= (__double2loint(w[m].x) | __double2loint(w[m].y)) != 0;
+        for (int m = 0; m < 8; ++m)
+            hi |= fx_high(0u, (unsigned)__double2loint(w[m].x) | (unsigned)__double2loint(w[m].y));
     }
     __syncthreads();
     atomicMax(ex + q, hi);
     __syncthreads();
-    unsigned E = ex[q] == 0u ? 1023u : ex[q] >> 20;   // a line of zeros fits any unit
+    unsigned E = fx_row_exponent(ex[q]);
     if (LOG2N >= 7 && fx_takes(E)) {
         unsigned s = 0;
 #pragma unroll

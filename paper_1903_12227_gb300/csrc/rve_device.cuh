@@ -665,8 +665,13 @@ __device__ __forceinline__ void hartley_row(double2 (&v)[8], double2* buf, int t
         for (int m = 0; m < 8; ++m)
             hi = max(hi, max((unsigned)__double2hiint(v[m].x) & 0x7FFFFFFFu,
                              (unsigned)__double2hiint(v[m].y) & 0x7FFFFFFFu));
+        if (hi == 0u) {   // zeros, or subnormals (which count as 1)
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+                hi |= fx_high(0u, (unsigned)__double2loint(v[m].x) | (unsigned)__double2loint(v[m].y));
+        }
     }
-    unsigned E = team_max<T>(hi, scratch, bar) >> 20;
+    unsigned E = fx_row_exponent(team_max<T>(hi, scratch, bar));
     bool fixed = !active || fx_takes(E);
     if (T < 32) fixed = __all_sync(0xffffffffu, fixed);
     if (fixed) {
