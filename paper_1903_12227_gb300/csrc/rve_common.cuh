@@ -149,6 +149,10 @@ __device__ __forceinline__ V stencil_apply(const CellsT<typename ScalarOf<V>::T>
 template <int SCHEME> __host__ __device__ constexpr double row_scale() { return SCHEME == 0 ? 6.0 : 2.0; }
 template <int SCHEME> __device__ __forceinline__ constexpr double row_centre() { return SCHEME == 0 ? 4.0 : 2.0; }
 struct StencilRow { double c, n, w, e, s, mm, m0, om, oo; };   // edges and corners without their signs
+template <int SCHEME> __device__ __forceinline__ StencilRow over_8(const StencilRow& r) {   // (c may have overflowed)
+    constexpr double k = 0.125;
+    return {k * row_centre<SCHEME>() * (r.n + r.s), k * r.n, k * r.w, k * r.e, k * r.s, k * r.mm, k * r.m0, k * r.om, k * r.oo};
+}
 
 constexpr int ROW_STRIDE = 10;   // doubles per table entry (16-byte loads, two-way conflicts at most)
 constexpr int ROW_TABLE = 16 * ROW_STRIDE;

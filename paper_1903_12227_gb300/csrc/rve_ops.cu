@@ -137,8 +137,14 @@ __global__ void __launch_bounds__(STIFF_THREADS) k_stiffness(const __grid_consta
         V m0 = at(i0, jm), m1 = at(i0, j), m2 = at(i0, jp);
         auto row = [&](const StencilRow& w, int i, const V& d0, const V& d1, const V& d2, auto doubled) {
             constexpr double IK = 1.0 / row_scale<SCHEME>();
-            const V q = apply_row<SCHEME, decltype(doubled)::value>(w, u0, u1, u2, m0, m1, m2, d0, d1, d2);
-            yb[((int64_t)i << lg) + j] = make_double2(IK * q.x, IK * q.y);
+            V q = apply_row<SCHEME, decltype(doubled)::value>(w, u0, u1, u2, m0, m1, m2, d0, d1, d2);
+            q = make_double2(IK * q.x, IK * q.y);
+            // K A x overflows where A x need not: again with the weights over 8
+            if (max((unsigned)__double2hiint(q.x) & 0x7FFFFFFFu, (unsigned)__double2hiint(q.y) & 0x7FFFFFFFu) >= 0x7FF00000u) {
+                q = apply_row<SCHEME, decltype(doubled)::value>(over_8<SCHEME>(w), u0, u1, u2, m0, m1, m2, d0, d1, d2);
+                q = make_double2(8.0 * IK * q.x, 8.0 * IK * q.y);
+            }
+            yb[((int64_t)i << lg) + j] = q;
             u0 = m0; u1 = m1; u2 = m2;
             m0 = d0; m1 = d1; m2 = d2;
         };
