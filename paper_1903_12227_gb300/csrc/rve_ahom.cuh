@@ -163,7 +163,7 @@ __device__ __forceinline__ void a_hom_tile(const RDesc& d, int64_t tile, CoefSrc
 // grids, so that one realization alone spreads over the chip.  By the grid's own
 // size: the tiles are summed one by one, and A_hom has to be the same bits alone
 // and in any batch.
-__host__ __device__ constexpr int a_hom_cells(int n) { return n <= 128 ? 64 : n <= 256 ? 256 : AHOM_TILE; }
+__host__ __device__ constexpr int a_hom_cells(int n) { return n <= 128 ? 64 : n <= 256 ? 512 : AHOM_TILE; }
 
 // Rows of a strip of a_hom_strip: min(n, AHOM_STRIP / n) rows of n cells.
 constexpr int AHOM_STRIP = 8192;
@@ -269,6 +269,8 @@ __device__ __forceinline__ void a_hom_tile_dd(const RDesc& d, int64_t tile, int 
             const uint32_t w = __ldg(cs.mask + d.word_off + (cidx >> 5));
             a = ((w >> (cidx & 31)) & 1u) ? d.a_incl : d.a_matrix;
         }
+        // (the first cell of a thread: 0 + v, without the additions)
+        auto add = [&](ddouble s, ddouble v) { return t < (int)blockDim.x ? v : dd_add(s, v); };
         const double2 r00 = at(i, j), r01 = at(i, j + 1), r10 = at(i + 1, j), r11 = at(i + 1, j + 1);
         ddouble w[2][3];   // a, b, c of the correctors
 #pragma unroll
@@ -283,7 +285,7 @@ __device__ __forceinline__ void a_hom_tile_dd(const RDesc& d, int64_t tile, int 
         if (FLUX) {   // P_11, P_12, P_21, P_22 over 3h (lumped h)
             acc[0] = dd_add(acc[0], a);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) acc[(4 + k) % NP] = dd_add(acc[(4 + k) % NP], dd_mul(w[k & 1][k >> 1], a));
+            for (int k = 0; k < 4; ++k) acc[(4 + k) % NP] = add(acc[(4 + k) % NP], dd_mul(w[k & 1][k >> 1], a));
         }
         w[0][0] = dd_add(w[0][0], 2.0 * h);   // v_i = xi_i + u_i
         w[1][1] = dd_add(w[1][1], 2.0 * h);
@@ -292,7 +294,7 @@ __device__ __forceinline__ void a_hom_tile_dd(const RDesc& d, int64_t tile, int 
             const int x = k == 2 ? 1 : 0, y = k == 0 ? 0 : 1;
             const ddouble ab = dd_add(dd_mul(w[x][0], w[y][0]), dd_mul(w[x][1], w[y][1]));
             const ddouble e = dd_add(SCHEME == 0 ? dd_mul(ab, 1.5) : dd_scale2(ab, 0.5), dd_mul(w[x][2], w[y][2]));
-            acc[E0 + k] = dd_add(acc[E0 + k], dd_mul(e, a));
+            acc[E0 + k] = add(acc[E0 + k], dd_mul(e, a));
         }
     }
     if (FLUX) {

@@ -85,7 +85,7 @@ __device__ __forceinline__ V ldv(const V* __restrict__ x, const RDesc& d, int i,
 // stay in FP32 -- through double, as the cell accessor returns them, every node
 // cost four conversions on the FP64 pipe -- and the kernel is bound by memory:
 // 96 x 512^2 nodes 250 -> 96 us.  FP64: bound by the FP64 pipe (StencilRow);
-// 11 x 1024^2 nodes, explicit cells 629 -> 570 us.
+// 11 x 1024^2 nodes, explicit cells 629 -> 566 us.
 constexpr int STIFF_THREADS = 256;
 template <typename V> __host__ __device__ constexpr int stiff_cols(int n) {   // columns of a block
     return n < (int)(4096 / sizeof(V)) ? n : (int)(4096 / sizeof(V));
