@@ -160,9 +160,10 @@ __device__ __forceinline__ void a_hom_tile(const RDesc& d, int64_t tile, CoefSrc
 }
 
 // Cells of an FP64 tile: one to four per thread of 64 to 256, fewer on small
-// grids, so that one realization alone spreads over the chip.  By the grid's own
-// size: the tiles are summed one by one, and A_hom has to be the same bits alone
-// and in any batch.
+// grids, so that one realization alone spreads over the chip (a call on one 256^2
+// grid: 113 us, 132 with 256 cells; on 500 64^2 grids 2.1 ms, 1.8 with 1024 cells
+// and less exact sums).  By the grid's own size: the tiles are summed one by one,
+// and A_hom has to be the same bits alone and in any batch.
 __host__ __device__ constexpr int a_hom_cells(int n) { return n <= 128 ? 64 : n <= 256 ? 512 : AHOM_TILE; }
 
 // Rows of a strip of a_hom_strip: min(n, AHOM_STRIP / n) rows of n cells.
@@ -240,8 +241,8 @@ __device__ __forceinline__ void a_hom_strip(const RDesc& d, int strip, CoefSrc c
 // plain double took 390 operations per cell instead of 470, but the error of
 // A + A_lo was 1.1 to 1.4 times as large (rms against 113 bits, n = 32; this
 // form's is that of the six products).  Calls of 1024^2: energy form 2.81 ms as
-// six products, 0.95 in that plain double, 1.08 now; with the flux form 2.90 ->
-// 1.39 ms (its eight sums were reduced by a butterfly each).
+// six products, 0.95 in that plain double, 1.05 now; with the flux form 2.90 ->
+// 1.32 ms (its eight sums were reduced by a butterfly each).
 // Partials out[2k], out[2k+1] = (hi, lo) of a_hom_tile's sums (k = 1, 2, 3 alone
 // without FLUX), the same bits with and without FLUX; `red` holds 8 x (FLUX ? 8 :
 // 4) ddouble (shared).
