@@ -42,7 +42,6 @@ constexpr int CHUNK = 96;
 struct DescChunk {
     int32_t count;
     int32_t start[CHUNK + 1];   // prefix sum of the launch's work units
-    int32_t real[CHUNK];        // index in the batch
     RDesc d[CHUNK];
 };
 

@@ -307,6 +307,7 @@ __global__ void __cluster_dims__(CHEB_CTAS, 1, 1) __launch_bounds__(32 * (CHEB_W
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (int)cl.block_rank(), b = blockIdx.x / CHEB_CTAS;
     const RDesc& d = ch.d[b];
+    if (d.n > CHEB_MAX_N) return;   // the whole cluster: k_cheb
     const int n = d.n, m = n - 1, lg = d.log2n, R = n / CHEB_CTAS, r0 = rank * R;
     const int tid = threadIdx.x, lane = tid & 31;
     const int rows = R * n;
@@ -397,7 +398,7 @@ __global__ void __cluster_dims__(CHEB_CTAS, 1, 1) __launch_bounds__(32 * (CHEB_W
                 for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
                 const double nc = __shfl_down_sync(0xffffffffu, x, 2);   // lanes 0, 1
                 if (lane < 2) {
-                    double* mb = mu + ((int64_t)ch.real[b] * 2 + lane) * K;
+                    double* mb = mu + ((int64_t)b * 2 + lane) * K;
                     if (q == 0) { mu0 = x; mu1 = nc; }
                     if (2 * q < K) mb[2 * q] = q == 0 ? x : 2.0 * x - mu0;
                     if (2 * q + 1 < K) mb[2 * q + 1] = q == 0 ? nc : 2.0 * nc - mu1;
@@ -415,12 +416,13 @@ __global__ void k_cheb_moments(const __grid_constant__ DescChunk ch, const doubl
     const int b = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (b >= ch.count) return;
     const int t0 = ch.start[b], nt = ch.start[b + 1] - t0;
+    if (nt == 0) return;   // a small grid: k_cheb_cluster
     double s[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) s[q] = warp_sum_array(part + (int64_t)t0 * 4 + q, nt, 4);
     if ((threadIdx.x & 31) != 0) return;
     for (int c = 0; c < 2; ++c) {
-        double* m = mu + ((int64_t)ch.real[b] * 2 + c) * K;
+        double* m = mu + ((int64_t)b * 2 + c) * K;
         const double cc = s[c], nc = s[2 + c];
         const double e = (k == 0) ? cc : 2.0 * cc - m[0];
         const double o = (k == 0) ? nc : 2.0 * nc - m[1];
@@ -538,7 +540,6 @@ static cudaError_t for_chunks(const Plan& p, UnitsFn units, LaunchFn fn) {
         ch.start[0] = 0;
         for (int k = 0; k < ch.count; ++k) {
             ch.d[k] = p.desc[b0 + k];
-            ch.real[k] = b0 + k;
             ch.start[k + 1] = ch.start[k] + (int32_t)units(ch.d[k]);
         }
         for (int k = ch.count + 1; k <= CHUNK; ++k) ch.start[k] = ch.start[ch.count];
@@ -643,46 +644,33 @@ cudaError_t launch_cheb(const Plan& p, void* ws, const uint32_t* mask, const dou
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_cheb_cluster<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
     if (e != cudaSuccess) return e;
-    return for_chunks(p, node_tiles, [&](const DescChunk& all, int) {
-        // the form by each grid's own size (the two round differently)
-        DescChunk ch = all;
-        ch.count = 0;
+    // the form by each grid's own size (the two round differently)
+    auto step_tiles = [](const RDesc& d) { return d.n <= CHEB_MAX_N ? (int64_t)0 : node_tiles(d); };
+    return for_chunks(p, step_tiles, [&](const DescChunk& ch, int first_real) {
+        double* m = mu + (int64_t)first_real * 2 * K;
         int maxn = 0;
-        for (int k = 0; k < all.count; ++k) {
-            if (all.d[k].n > CHEB_MAX_N) continue;
-            maxn = std::max(maxn, all.d[k].n);
-            ch.real[ch.count] = all.real[k];
-            ch.d[ch.count++] = all.d[k];
-        }
-        if (ch.count > 0) {   // two vectors of a realization fit a cluster's shared memory
+        for (int k = 0; k < ch.count; ++k)
+            if (ch.d[k].n <= CHEB_MAX_N) maxn = std::max(maxn, ch.d[k].n);
+        if (maxn > 0) {   // two vectors of a realization fit a cluster's shared memory
             const size_t smem = 2 * sizeof(double2) * (size_t)maxn * maxn / CHEB_CTAS;
             auto kern = scheme == RVE_Q1_LUMPED ? k_cheb_cluster<1> : k_cheb_cluster<0>;
-            kern<<<ch.count * CHEB_CTAS, 32 * (CHEB_WARPS + 1), smem, s>>>(ch, cs, a0, a1, steps, K, v, mu);
+            kern<<<ch.count * CHEB_CTAS, 32 * (CHEB_WARPS + 1), smem, s>>>(ch, cs, a0, a1, steps, K, v, m);
             const cudaError_t ce = cudaGetLastError();
-            if (ce != cudaSuccess || ch.count == all.count) return ce;
+            if (ce != cudaSuccess) return ce;
         }
-        ch.count = 0;
-        int64_t from = 0, to = 0;   // nodes of a run of realizations whose w_0 is still to copy
-        auto copy = [&]() -> cudaError_t {
-            if (from == to) return cudaSuccess;
-            return cudaMemcpyAsync(wb + from, v + 2 * from, sizeof(double2) * (size_t)(to - from),
-                                   cudaMemcpyDeviceToDevice, s);
-        };
-        for (int k = 0; k < all.count; ++k) {
-            const RDesc& d = all.d[k];
-            if (d.n <= CHEB_MAX_N) continue;
-            if (d.node_off != to) {
-                const cudaError_t ce = copy();
+        for (int k = 0; k < ch.count;) {   // w_0 of every run of large grids
+            int e = k;
+            while (e < ch.count && ch.d[e].n > CHEB_MAX_N) ++e;
+            if (e > k) {
+                const int64_t from = ch.d[k].node_off;
+                const int64_t to = ch.d[e - 1].node_off + (int64_t)ch.d[e - 1].n * ch.d[e - 1].n;
+                const cudaError_t ce = cudaMemcpyAsync(wb + from, v + 2 * from, sizeof(double2) * (size_t)(to - from),
+                                                       cudaMemcpyDeviceToDevice, s);
                 if (ce != cudaSuccess) return ce;
-                from = d.node_off;
             }
-            to = d.node_off + (int64_t)d.n * d.n;
-            ch.start[ch.count + 1] = ch.start[ch.count] + (int32_t)node_tiles(d);
-            ch.real[ch.count] = all.real[k];
-            ch.d[ch.count++] = d;
+            k = e + 1;
         }
-        const cudaError_t ce = copy();
-        if (ce != cudaSuccess) return ce;
+        if (ch.start[ch.count] == 0) return cudaSuccess;
         const int g = ch.start[ch.count];
         double2* cur = wb;    // w_k
         double2* oth = wa;    // in: w_{k-1}, out: w_{k+1}
@@ -691,7 +679,7 @@ cudaError_t launch_cheb(const Plan& p, void* ws, const uint32_t* mask, const dou
                 k_cheb<1><<<g, NODE_TILE, 0, s>>>(ch, cs, a0, a1, k == 0, cur, oth, part);
             else
                 k_cheb<0><<<g, NODE_TILE, 0, s>>>(ch, cs, a0, a1, k == 0, cur, oth, part);
-            k_cheb_moments<<<(ch.count + 7) / 8, 256, 0, s>>>(ch, part, k, K, mu);
+            k_cheb_moments<<<(ch.count + 7) / 8, 256, 0, s>>>(ch, part, k, K, m);
             note_launch(2);
             const cudaError_t le = cudaGetLastError();
             if (le != cudaSuccess) return le;
